@@ -375,8 +375,7 @@ int create_reg_batch(const hs_batch_job* jobs, size_t n_jobs, const hs_batch_opt
       }
       std::vector<int> ids;
       for (auto& pc : pieces) {
-        hs::q::fill_job(J.factors, *pc.second, J.psi, J.n_rhs);
-        pc.second->units_per_cta = 1;
+        hs::q::fill_job(J.factors, *pc.second, J.psi, J.n_rhs, 1);
         ids.push_back(int(P.pieces.size()));
         P.pieces.push_back(std::move(pc.second));
       }

@@ -18,6 +18,8 @@ constexpr int kMaxXDim = 6;         // log2 of the x-mask set size per factor
 constexpr int kMaxRuns = 6;         // contiguous bit runs describing a tile's local bits
 constexpr int kMaxSweepFactors = 64;
 constexpr int kMaxFusedDiags = 32;                 // factors with more diagonals use the plain kernel
+constexpr int kSMs = 152;                          // SMs of a GB300
+constexpr size_t kSmemPerSm = 228 * 1024;          // shared memory of an SM, 1 KiB of it per resident CTA reserved
 constexpr size_t kSweepSmemMax = 227 * 1024;       // opt-in shared memory per CTA
 constexpr size_t kSweepSmemDefault = 112 * 1024;   // two sweep CTAs per SM
 constexpr int kMaxVtBits = 8;       // qubits a factor's terms may touch for a value table

@@ -87,10 +87,23 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     const size_t first_op = ops.size();
     const Group& G = p.groups[g];
     if ((G.span & ~uint64_t(local_mask)) != 0) return fail("factor flips outside the tile");
+    // XX, YY and ZZ of one qubit pair with one coefficient, next to each other
+    // in any order, act as one BOND (static sets: a drive may part the three).
+    auto bond_at = [&](int j) {
+      if (steps || f->bin.coeff1 || j < G.first || j + 3 > G.last) return false;
+      const uint64_t u = p.x[j] | p.z[j];
+      int kinds = 0;
+      for (int k = j; k < j + 3; ++k) {
+        if ((p.x[k] | p.z[k]) != u || (p.x[k] & ~u) || p.coeff[k] != p.coeff[j]) return false;
+        if ((p.x[k] && p.x[k] != u) || (p.z[k] && p.z[k] != u)) return false;
+        kinds |= p.x[k] ? (p.z[k] ? 2 : 1) : 4;
+      }
+      return __builtin_popcountll(u) == 2 && kinds == 7;
+    };
     // A factor of several terms with a value table of at most two slots (a
-    // Heisenberg bond) is read from its table; a single term is cheaper as
-    // its rotation.
-    if (G.last - G.first > 1 && G.vt0 >= 0 && G.nslot >= 1 && G.nslot <= 2 && G.vt_n <= kMaxVt) {
+    // bond whose couplings differ) is read from its table; a single term is
+    // cheaper as its rotation, and three equal ones as a BOND.
+    if (!(G.last - G.first == 3 && bond_at(G.first)) && G.last - G.first > 1 && G.vt0 >= 0 && G.nslot >= 1 && G.nslot <= 2 && G.vt_n <= kMaxVt) {
       const uint32_t u = G.nslot == 2 ? p.slot_u[G.slot0 + 1] : 0u;
       if (__builtin_popcount(loc(u)) <= 2) {
         // (value tables hold one step's values: not in a sweep that spans steps)
@@ -103,6 +116,15 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     const int cnt = G.last - G.first;
     for (int q = 0; q < cnt; ++q) {
       const int j = G.dir > 0 ? G.first + q : G.last - 1 - q;
+      if (bond_at(G.dir > 0 ? j : j - 2)) {
+        if (!run.empty()) {
+          ops.push_back(HOp{OP_PHASE, g, -1, run, 0});
+          run.clear();
+        }
+        ops.push_back(HOp{OP_BOND, g, G.dir > 0 ? j : j - 2, {}, loc(p.x[j] | p.z[j])});
+        q += 2;
+        continue;
+      }
       if (p.x[j] == 0) {
         run.push_back(j);
         continue;
@@ -136,10 +158,20 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     for (int b = lane_lo; b < lane_hi && b < T && __builtin_popcount(R) < B; ++b) R |= 1u << b;
     return R;
   };
+  // A run of X-type rotations (y = 0, z = 0) commutes: those that fit the
+  // register bits in effect go first, so that a run after a phase undoes the
+  // layouts of the run before it (a MaxCut sweep makes 4 layout changes, not 5).
+  auto x_type = [&](const HOp& h) { return h.type == OP_ROT && p.z[h.term] == 0; };
   std::vector<uint32_t> lay_of(ops.size(), 0);
   uint32_t cur = 0;
   bool have = false;
   for (size_t i = 0; i < ops.size(); ++i) {
+    if (have && x_type(ops[i]) && (i == 0 || !x_type(ops[i - 1]))) {
+      size_t e = i;
+      while (e < ops.size() && x_type(ops[e])) ++e;
+      std::stable_partition(ops.begin() + i, ops.begin() + e,
+                            [&](const HOp& h) { return ((h.need | pin) & ~cur) == 0; });
+    }
     const bool reg = ops[i].type != OP_PHASE;
     if (reg && (!have || ((ops[i].need | pin) & ~cur))) {
       uint32_t R = ops[i].need | pin;
@@ -193,8 +225,8 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     warp_pos[li] = w;
   }
   std::map<std::pair<uint32_t, std::vector<int>>, int> lay_id;
-  std::map<int, int> rot_id, tab_id;
-  std::map<std::tuple<int, int, uint32_t, int>, int> phase_id;  // (factor, first term of the run, layout, relative step)
+  std::map<int, int> rot_id, tab_id, bond_id;
+  std::map<std::tuple<int, int, int, int>, int> phase_id;  // (factor, first term of the run, layout, relative step)
   auto add_layout = [&](uint32_t R, const std::vector<int>& wpos) -> int {
     const auto key = std::make_pair(R, wpos);
     auto it = lay_id.find(key);
@@ -203,12 +235,16 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     Layout& L = a.lay[a.n_lay];
     L = Layout();
     L.reg = R;
+    const int in_chunk = c64 ? 1 : 0;  // register bits inside a 16-byte chunk
     int i = 0;
     for (uint32_t t = R; t; t &= t - 1u, ++i) {
-      const int rp = __builtin_ctz(t);
-      const uint32_t bit = 1u << rp;
-      L.qoff[i] = (c64 && rp == 0) ? 0u : swz(c64 ? (bit >> 1) : bit);
-      L.goff[i] = glob(bit);
+      const uint32_t bit = t & (0u - t);
+      if (i < in_chunk) {
+        L.g0 = glob(bit);
+      } else {
+        L.qoff[i - in_chunk] = swz(c64 ? (bit >> 1) : bit);
+        L.goff[i - in_chunk] = glob(bit);
+      }
     }
     // Lanes: the thread bits that are not warp bits, three whose chunk bits
     // differ mod 3 first (the eight threads of a quarter-warp then hit
@@ -238,14 +274,11 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
       if (std::find(wpos.begin(), wpos.end(), b) == wpos.end()) W.push_back(c64 ? b - 1 : b);
     if (W.size() < 5) return -1;
     for (int k = 0; k < 5; ++k) L.wlo[k] = int8_t(W[k]);
-    const int nj = 1 << (B - (c64 ? 1 : 0));
-    if (int(W.size()) != 5 + (B - (c64 ? 1 : 0))) return -1;
-    for (int mm = 0; mm < nj; ++mm) {
-      uint32_t c = 0;
-      for (int k = 0; k < B - (c64 ? 1 : 0); ++k)
-        if ((mm >> k) & 1) c |= 1u << W[5 + k];
-      L.mswz[mm] = swz(c);
-      L.mglob[mm] = glob(c64 ? (c << 1) : c);
+    if (int(W.size()) != 5 + (B - in_chunk)) return -1;
+    for (int k = 0; k < B - in_chunk; ++k) {
+      const uint32_t c = 1u << W[5 + k];
+      L.mswz[k] = swz(c);
+      L.mglob[k] = glob(c64 ? (c << 1) : c);
     }
     lay_id[key] = a.n_lay;
     return a.n_lay++;
@@ -253,7 +286,7 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
   auto reg_coords = [&](uint32_t lmask, uint32_t R) { return pext32(lmask & R, R); };
 
   uint32_t emitted = 0xffffffffu;  // no layout yet
-  int seq_i = -1;
+  int seq_i = -1, cur_li = -1;
   std::vector<PClass> cls;
   std::vector<PTerm> pts;
   for (size_t i = 0; i < ops.size(); ++i) {
@@ -263,6 +296,7 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
       ++seq_i;
       const int li = add_layout(R, warp_pos[seq_i]);
       if (li < 0) return fail("too many register layouts");
+      cur_li = li;
       if (a.n_ops >= kMaxOps) return fail("too many ops");
       Op& o = a.ops[a.n_ops++];
       o = Op();
@@ -297,6 +331,16 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
       }
       o.idx = int16_t(ti);
       o.ku = uint8_t(reg_coords(h.need, R));
+    } else if (h.type == OP_BOND) {
+      const int key = G.kind * m + h.term;
+      auto it = bond_id.find(key);
+      if (it == bond_id.end()) {
+        if (a.n_bond >= kMaxBond) return fail("too many bonds");
+        a.bond[a.n_bond] = key;
+        it = bond_id.emplace(key, a.n_bond++).first;
+      }
+      o.idx = int16_t(it->second);
+      o.ku = uint8_t(reg_coords(h.need, R));
     } else if (h.type == OP_ROT || (h.type == OP_PHASE && h.terms.size() == 1)) {
       // (a run of one diagonal term is a diagonal rotation, DROT)
       const int term = h.type == OP_ROT ? h.term : h.terms[0];
@@ -323,7 +367,7 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
       o.zrest = uint32_t(z & ~uint64_t(local_mask));
       o.flags = uint8_t((x != 0 && z == 0 ? 1 : 0) | (((y + 3) & 3) << 1));
     } else {
-      const auto key = std::make_tuple(h.g, h.terms.front(), R, h.rs);
+      const auto key = std::make_tuple(h.g, h.terms.front(), cur_li, h.rs);
       auto it = phase_id.find(key);
       int pi;
       if (it != phase_id.end()) {
@@ -411,6 +455,27 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
   a.n_pterm = int(pts.size());
   std::copy(cls.begin(), cls.end(), a.cls);
   std::copy(pts.begin(), pts.end(), a.pt);
+  for (int i = 0; i < a.n_ops; ++i)
+    if (a.ops[i].type == OP_LAYOUT) a.last_lay = i;  // the tile buffer's last reader
+  a.free_local = warp_pos.front() == warp_pos.back() ? 1 : 0;
+  // Factor slots: every phase its own while that leaves the tile's CTAs per SM
+  // (two with 64 KiB tiles), else shared ones.
+  const uint32_t eb = uint32_t(elem_bytes(f->dtype));
+  a.fac_keep = 1;
+  int n_shared = 0;
+  for (int i = 0; i < a.n_phase; ++i) {
+    const uint32_t mm = a.ph[i].mu_mask;
+    const int own = 1 + B + __builtin_popcount(B == 5 ? inside_patterns<5>(mm) : inside_patterns<4>(mm));
+    const int across = __builtin_popcount(B == 5 ? across_patterns<5>(mm) : across_patterns<4>(mm));
+    a.ph[i].fac0 = int16_t(a.n_fac);
+    a.n_fac += own + across;
+    n_shared = std::max(n_shared, own + (across ? 1 : 0));
+  }
+  if (qsweep_smem_bytes(a, f->dtype, B) > ((size_t(eb) << T) <= (size_t(64) << 10) ? kSweepSmemDefault : kSweepSmemMax)) {
+    a.fac_keep = 0;
+    a.n_fac = n_shared;
+    for (int i = 0; i < a.n_phase; ++i) a.ph[i].fac0 = 0;
+  }
   a.full = 0;
   for (int i = 0; i < a.n_ops; ++i)
     if (a.ops[i].type == OP_TAB || (a.ops[i].type == OP_ROT && !(a.ops[i].flags & 1))) a.full = 1;

@@ -1,27 +1,44 @@
 // Register-blocked tile sweep (see qsweep.h for the descriptor).
 //
-// One CTA evolves a tile of 2^T amplitudes of one state through every op of
-// the sweep:
+// One CTA evolves tiles of 2^T amplitudes of one state through every op of the
+// sweep:
 //   1. the tile is copied from HBM into shared memory with 16-byte cp.async
 //      copies (chunk c of the tile lands at the swizzled chunk swz(c));
 //   2. each thread reads its 2^B rows for the first register layout into
 //      registers and applies the ops: a factor whose flips lie in the
 //      register bits touches only registers; a LAYOUT op writes the rows back
 //      and reads them again for the next set of register bits;
-//   3. the rows go back through shared memory and out to HBM with coalesced
-//      16-byte stores.
+//   3. the rows go straight from registers to HBM in the last layout.
 // With T = 13 and B = 5 the tile is 64 KiB, the CTA has 256 threads, and a
-// step of the 24-qubit MaxCut instance (24 factors) takes two sweeps, each
-// reading and writing the states once.
+// step of the 24-qubit MaxCut instance (24 factors) takes one sweep.
+//
+// What bounds it: HBM (2 * s * N * R bytes per sweep) for few ops per
+// amplitude, the FP32 pipe and the shared-memory path of the layout changes
+// for many; but before either, instruction delivery.  The kernel is an
+// interpreter of fully unrolled op bodies, and with scalar complex arithmetic,
+// a phase body with a sincospi per register pattern and four store bodies its
+// warps stalled on instruction fetch more than on anything else (2.3 warps per
+// issue, instruction-cache hit rate 78%, 24-qubit sweep 2.09 ms).  So the
+// executed footprint is kept small: complex64 rows are held as pairs
+// (re0, re1), (im0, im1) of the two rows that differ in register bit 0, and
+// every op works on pairs with the two-element FP32 instructions (half the
+// instructions of the scalar form for the same operations), and the phase
+// factors are produced by one loop with one sincospi.  On the 24-qubit MaxCut
+// instance with 16 states a sweep went from 2.09 to 1.51 ms; a periodic
+// 22-qubit Heisenberg chain with 2 states (BOND ops) from 3.85 to 1.72 ms for
+// 20 steps.  Registers matter as much: the tiles leave little L1, so a spilled
+// register costs an L2 round trip (52 local loads per warp and tile made the
+// 1.51 ms sweep a 6.2 ms one).
 //
 // PHASE ops generate a diagonal run's values from (z_j, theta_j): with the
 // tile's fixed bits folded in, phi(r) = C0 + sum_m C_m chi_m(l), where m runs
 // over the distinct local parts of the z_j, chi_m(l) = (-1)^popcount(m & l)
-// and C_m sums +-theta_j (FP64, once per tile).  A thread's rows differ only
-// in their register bits, so phi over its 2^B rows is the Walsh-Hadamard
+// and C_m sums +-theta_j (units of pi, once per tile).  A thread's rows differ
+// only in their register bits, so phi over its 2^B rows is the Walsh-Hadamard
 // transform of the per-thread coefficients E[mu] = sum over classes with
-// register part mu of +-C_m; each row then takes exp(-i phi) (sincospi in
-// the bulk precision, with exp(-i C0) from an FP64 sincos per tile).
+// register part mu of +-C_m; each row takes a product of exp(-+ i pi E[mu]).
+// They do not depend on the state: a CTA runs up to kMaxRhsChunk states of a
+// tile back to back and computes them for the first one only.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,9 +64,6 @@ using sweep::grid_dependency_wait;
 using sweep::grid_launch_dependents;
 using sweep::pattern_fast;
 
-__device__ __forceinline__ void sincospi_r(float x, float* s, float* c) { sincospif(x, s, c); }
-__device__ __forceinline__ void sincospi_r(double x, double* s, double* c) { sincospi(x, s, c); }
-
 __device__ __forceinline__ int parity(uint32_t v) { return __popc(v) & 1; }
 
 __host__ __device__ constexpr int highest_bit(int v) {
@@ -58,12 +72,53 @@ __host__ __device__ constexpr int highest_bit(int v) {
   return v ? (1 << h) : 0;
 }
 
-
-// (re, im) * (c, s) helpers.
+// (re, im) * (bx, by).
 template <typename T2, typename R>
 __device__ __forceinline__ T2 cmul(T2 a, R bx, R by) {
   return T2{fma(a.x, bx, -a.y * by), fma(a.x, by, a.y * bx)};
 }
+
+// v with its sign flipped where the lowest bit of s is set.
+__device__ __forceinline__ float flip_sign(float v, uint32_t s) {
+  return __uint_as_float(__float_as_uint(v) ^ (s << 31));
+}
+__device__ __forceinline__ double flip_sign(double v, uint32_t s) { return (s & 1u) ? -v : v; }
+
+// ---------------------------------------------------------------------------
+// A thread's 2^B rows.  complex64: rows 2j and 2j + 1 share the pairs re[j]
+// and im[j]; complex128: row by row.
+// ---------------------------------------------------------------------------
+template <typename R, int B>
+struct Rows;
+
+template <int B>
+struct Rows<float, B> {
+  static constexpr int NP = 1 << (B - 1);
+  float2 re[NP], im[NP];
+  __device__ __forceinline__ float2 get(int k) const {
+    return (k & 1) ? make_float2(re[k >> 1].y, im[k >> 1].y) : make_float2(re[k >> 1].x, im[k >> 1].x);
+  }
+  __device__ __forceinline__ void set(int k, float2 v) {
+    if (k & 1) {
+      re[k >> 1].y = v.x;
+      im[k >> 1].y = v.y;
+    } else {
+      re[k >> 1].x = v.x;
+      im[k >> 1].x = v.y;
+    }
+  }
+};
+
+template <int B>
+struct Rows<double, B> {
+  double2 x[1 << B];
+  __device__ __forceinline__ double2 get(int k) const { return x[k]; }
+  __device__ __forceinline__ void set(int k, double2 v) { x[k] = v; }
+};
+
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // ---------------------------------------------------------------------------
 // ROT: x <- (cos I - i sin P_j) x for one term whose flips are the register
@@ -77,56 +132,119 @@ __device__ __forceinline__ T2 cmul(T2 a, R bx, R by) {
 // scale, and an odd k swaps the partner rows (flip_pairs) at the end of the
 // op, so the rotation itself has no data-dependent branch.
 // ---------------------------------------------------------------------------
-template <typename R, int NR, int KU>
-__device__ __forceinline__ void rot_tan(typename C2<R>::T (&x)[NR], R t) {
-  using T2 = typename C2<R>::T;
+template <int KU, int B>
+__device__ __forceinline__ void rot_tan(Rows<float, B>& x, float t) {
+  constexpr int NP = Rows<float, B>::NP;
+  constexpr int JU = KU >> 1, HB = highest_bit(JU);
+  if constexpr ((KU & 1) == 0) {
+    const float2 tp = dup(t), tn = dup(-t);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      if (j & HB) continue;
+      const int j2 = j ^ JU;
+      const float2 r1 = x.re[j], m1 = x.im[j], r2 = x.re[j2], m2 = x.im[j2];
+      x.re[j] = fma2(tp, m2, r1);
+      x.im[j] = fma2(tn, r2, m1);
+      x.re[j2] = fma2(tp, m1, r2);
+      x.im[j2] = fma2(tn, r1, m2);
+    }
+  } else {
+    // The partner sits in the other half of a pair.
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      if (j & HB) continue;
+      const int j2 = j ^ JU;
+      const float2 r1 = x.re[j], m1 = x.im[j], r2 = x.re[j2], m2 = x.im[j2];
+      x.re[j] = make_float2(fmaf(t, m2.y, r1.x), fmaf(t, m2.x, r1.y));
+      x.im[j] = make_float2(fmaf(-t, r2.y, m1.x), fmaf(-t, r2.x, m1.y));
+      if constexpr (JU != 0) {
+        x.re[j2] = make_float2(fmaf(t, m1.y, r2.x), fmaf(t, m1.x, r2.y));
+        x.im[j2] = make_float2(fmaf(-t, r1.y, m2.x), fmaf(-t, r1.x, m2.y));
+      }
+    }
+  }
+}
+
+template <int KU, int B>
+__device__ __forceinline__ void rot_tan(Rows<double, B>& x, double t) {
   constexpr int HB = highest_bit(KU);
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
+  for (int k = 0; k < (1 << B); ++k) {
     if (k & HB) continue;
     const int k2 = k ^ KU;
-    const T2 b1 = x[k], b2 = x[k2];
-    x[k] = T2{fma(t, b2.y, b1.x), fma(-t, b2.x, b1.y)};
-    x[k2] = T2{fma(t, b1.y, b2.x), fma(-t, b1.x, b2.y)};
+    const double2 b1 = x.x[k], b2 = x.x[k2];
+    x.x[k] = make_double2(fma(t, b2.y, b1.x), fma(-t, b2.x, b1.y));
+    x.x[k2] = make_double2(fma(t, b1.y, b2.x), fma(-t, b1.x, b2.y));
   }
 }
 
-template <typename R, int NR, int KU>
-__device__ __forceinline__ void flip_pairs(typename C2<R>::T (&x)[NR]) {
-  using T2 = typename C2<R>::T;
+template <typename R, int KU, int B>
+__device__ __forceinline__ void flip_pairs(Rows<R, B>& x) {
   constexpr int HB = highest_bit(KU);
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
+  for (int k = 0; k < (1 << B); ++k) {
     if (k & HB) continue;
-    const T2 b = x[k];
-    x[k] = x[k ^ KU];
-    x[k ^ KU] = b;
+    const auto b = x.get(k);
+    x.set(k, x.get(k ^ KU));
+    x.set(k ^ KU, b);
   }
 }
 
-template <typename R, int NR, int KU>
-__device__ __forceinline__ void rot_ku(typename C2<R>::T (&x)[NR], R c, R s, bool fast, int q, uint32_t zk,
-                                       int sb, bool flip) {
+template <typename R, int KU, int B>
+__device__ __forceinline__ void rot_ku(Rows<R, B>& x, R c, R s, bool fast, int q, uint32_t zk, int sb, bool flip) {
   using T2 = typename C2<R>::T;
   constexpr int HB = highest_bit(KU);
   if (fast) {
-    rot_tan<R, NR, KU>(x, c);
-    if (flip) flip_pairs<R, NR, KU>(x);
+    rot_tan<KU>(x, c);
+    if (flip) flip_pairs<R, KU>(x);
     return;
   }
   const R qx = (q == 0) ? s : (q == 2 ? -s : R(0));
   const R qy = (q == 1) ? s : (q == 3 ? -s : R(0));
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
+  for (int k = 0; k < (1 << B); ++k) {
     if (k & HB) continue;
     const int k2 = k ^ KU;
-    const T2 b1 = x[k], b2 = x[k2];
+    const T2 b1 = x.get(k), b2 = x.get(k2);
     // row k pairs with column k2 (sign of r_k2), row k2 with column k (sign of r_k)
     const R sk = (sb ^ parity(zk & uint32_t(k2))) ? R(-1) : R(1);
     const R sk2 = (sb ^ parity(zk & uint32_t(k))) ? R(-1) : R(1);
     const R ax = sk * qx, ay = sk * qy, bx = sk2 * qx, by = sk2 * qy;
-    x[k] = T2{fma(ax, b2.x, fma(-ay, b2.y, c * b1.x)), fma(ax, b2.y, fma(ay, b2.x, c * b1.y))};
-    x[k2] = T2{fma(bx, b1.x, fma(-by, b1.y, c * b2.x)), fma(bx, b1.y, fma(by, b1.x, c * b2.y))};
+    x.set(k, T2{fma(ax, b2.x, fma(-ay, b2.y, c * b1.x)), fma(ax, b2.y, fma(ay, b2.x, c * b1.y))});
+    x.set(k2, T2{fma(bx, b1.x, fma(-by, b1.y, c * b2.x)), fma(bx, b1.y, fma(by, b1.x, c * b2.y))});
+  }
+}
+
+// ---------------------------------------------------------------------------
+// BOND: rows (.., 0 1, ..) and (.., 1 0, ..) on the two register bits of KU
+// become a + w (b - a) and b - w (b - a); the other rows stay.
+// ---------------------------------------------------------------------------
+template <typename R, int KU, int B>
+__device__ __forceinline__ void bond_rows(Rows<R, B>& x, typename C2<R>::T w) {
+  using T2 = typename C2<R>::T;
+  constexpr int HB = highest_bit(KU), LB = KU ^ HB;
+  if constexpr (sizeof(R) == 4 && (KU & 1) == 0) {
+    constexpr int NP = 1 << (B - 1);
+    const float2 wx = dup(w.x), wy = dup(w.y), nx = dup(-w.x), ny = dup(-w.y), m1 = dup(-1.0f);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      if ((j & (HB >> 1)) || !(j & (LB >> 1))) continue;
+      const int j2 = j ^ (KU >> 1);
+      const float2 dr = fma2(m1, x.re[j], x.re[j2]), di = fma2(m1, x.im[j], x.im[j2]);
+      x.re[j] = fma2(wx, dr, fma2(ny, di, x.re[j]));
+      x.im[j] = fma2(wx, di, fma2(wy, dr, x.im[j]));
+      x.re[j2] = fma2(nx, dr, fma2(wy, di, x.re[j2]));
+      x.im[j2] = fma2(nx, di, fma2(ny, dr, x.im[j2]));
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < (1 << B); ++k) {
+      if ((k & HB) || !(k & LB)) continue;
+      const T2 a = x.get(k), b = x.get(k ^ KU);
+      const R dx = b.x - a.x, dy = b.y - a.y;
+      x.set(k, T2{fma(w.x, dx, fma(-w.y, dy, a.x)), fma(w.x, dy, fma(w.y, dx, a.y))});
+      x.set(k ^ KU, T2{fma(-w.x, dx, fma(w.y, dy, b.x)), fma(-w.x, dy, fma(-w.y, dx, b.y))});
+    }
   }
 }
 
@@ -135,10 +253,11 @@ __device__ __forceinline__ void rot_ku(typename C2<R>::T (&x)[NR], R c, R s, boo
 // row k's global index at the factor's support (p_k = pt ^ XOR of pr[i] over
 // the set bits i of k: the pattern map is linear over XOR).
 // ---------------------------------------------------------------------------
-template <typename R, int NR, int B, int KU>
-__device__ __forceinline__ void tab_ku(typename C2<R>::T (&x)[NR], const typename C2<R>::T* tb, int ns,
-                                       uint32_t pt, const uint32_t (&pr)[B]) {
+template <typename R, int B, int KU>
+__device__ __forceinline__ void tab_ku(Rows<R, B>& x, const typename C2<R>::T* tb, int ns, uint32_t pt,
+                                       const uint32_t (&pr)[B]) {
   using T2 = typename C2<R>::T;
+  constexpr int NR = 1 << B;
   constexpr int HB = KU ? highest_bit(KU) : 0;
   // Pattern of register row k: pt ^ XOR of pr[i] over the set bits i of k.
   auto pat = [&](int k) {
@@ -152,113 +271,115 @@ __device__ __forceinline__ void tab_ku(typename C2<R>::T (&x)[NR], const typenam
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
       const T2 v0 = tb[pat(k) * uint32_t(ns)];
-      x[k] = T2{fma(v0.x, x[k].x, -v0.y * x[k].y), fma(v0.x, x[k].y, v0.y * x[k].x)};
+      x.set(k, cmul<T2, R>(x.get(k), v0.x, v0.y));
     }
   } else {
-  // Two slots: a row's entries (r, r) and (r, r ^ u) sit side by side in the
-  // table, one 2 * sizeof(T2)-byte load.
+    // Two slots: a row's entries (r, r) and (r, r ^ u) sit side by side in the
+    // table, one 2 * sizeof(T2)-byte load.
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
-    if (k & HB) continue;
-    const int k2 = k ^ KU;
-    T2 a0, a1, c0, c1;
-    if constexpr (sizeof(T2) == 8) {
-      const float4 va = *reinterpret_cast<const float4*>(tb + pat(k) * 2u);
-      const float4 vc = *reinterpret_cast<const float4*>(tb + pat(k2) * 2u);
-      a0 = T2{va.x, va.y};
-      a1 = T2{va.z, va.w};
-      c0 = T2{vc.x, vc.y};
-      c1 = T2{vc.z, vc.w};
-    } else {
-      const T2* va = tb + pat(k) * 2u;
-      const T2* vc = tb + pat(k2) * 2u;
-      a0 = va[0];
-      a1 = va[1];
-      c0 = vc[0];
-      c1 = vc[1];
+    for (int k = 0; k < NR; ++k) {
+      if (k & HB) continue;
+      const int k2 = k ^ KU;
+      T2 a0, a1, c0, c1;
+      if constexpr (sizeof(T2) == 8) {
+        const float4 va = *reinterpret_cast<const float4*>(tb + pat(k) * 2u);
+        const float4 vc = *reinterpret_cast<const float4*>(tb + pat(k2) * 2u);
+        a0 = T2{va.x, va.y};
+        a1 = T2{va.z, va.w};
+        c0 = T2{vc.x, vc.y};
+        c1 = T2{vc.z, vc.w};
+      } else {
+        const T2* va = tb + pat(k) * 2u;
+        const T2* vc = tb + pat(k2) * 2u;
+        a0 = va[0];
+        a1 = va[1];
+        c0 = vc[0];
+        c1 = vc[1];
+      }
+      const T2 b1 = x.get(k), b2 = x.get(k2);
+      T2 r1, r2;
+      r1.x = fma(a0.x, b1.x, fma(-a0.y, b1.y, fma(a1.x, b2.x, -a1.y * b2.y)));
+      r1.y = fma(a0.x, b1.y, fma(a0.y, b1.x, fma(a1.x, b2.y, a1.y * b2.x)));
+      r2.x = fma(c0.x, b2.x, fma(-c0.y, b2.y, fma(c1.x, b1.x, -c1.y * b1.y)));
+      r2.y = fma(c0.x, b2.y, fma(c0.y, b2.x, fma(c1.x, b1.y, c1.y * b1.x)));
+      x.set(k, r1);
+      x.set(k2, r2);
     }
-    const T2 b1 = x[k], b2 = x[k2];
-    T2 r1, r2;
-    r1.x = fma(a0.x, b1.x, fma(-a0.y, b1.y, fma(a1.x, b2.x, -a1.y * b2.y)));
-    r1.y = fma(a0.x, b1.y, fma(a0.y, b1.x, fma(a1.x, b2.y, a1.y * b2.x)));
-    r2.x = fma(c0.x, b2.x, fma(-c0.y, b2.y, fma(c1.x, b1.x, -c1.y * b1.y)));
-    r2.y = fma(c0.x, b2.y, fma(c0.y, b2.x, fma(c1.x, b1.y, c1.y * b1.x)));
-    x[k] = r1;
-    x[k2] = r2;
-  }
   }
 }
 
-// ROTN: commuting X rotations on distinct single register bits (tan form,
-// see ROT), the slot of register bit i in byte i of (zthr, zrest).  The full
-// run and the run without bit 0 are straight-line bodies; any other run tests
-// its bits.  The odd-k swaps follow the whole run (every factor of the run is
-// a function of its own X, so they commute).
+// An op's coefficients: ROTN the tan(theta') of register bits 0 .. 4, ROT and
+// DROT (cos, sin) or (tan, 0), BOND w; `swap` the register bits (ROTN) or the
+// flag (ROT) of odd quarter turns.
+template <typename R>
+struct alignas(16) Coef {
+  R v[5];
+  uint32_t swap;
+  uint32_t pad[sizeof(R) == 4 ? 2 : 1];
+};
+
+// ROTN: commuting X rotations on distinct single register bits (tan form, see
+// ROT), the slot of register bit i in byte i of (zthr, zrest).  The rows of
+// one rotation change register in pairs, so a body that ends in a branch pays
+// a move per row; the run over all bits above bit 0 (a full layout of single
+// flips) is therefore one straight-line body (24-qubit MaxCut: 87.5 ms with a
+// branch per bit).  The odd-k swaps follow the whole run (every factor of the
+// run is a function of its own X, so they commute).
 __device__ __forceinline__ int rotn_slot(const Op& op, int i) {
   return int((i < 4 ? (op.zthr >> (8 * i)) : (op.zrest >> (8 * (i - 4)))) & 0xffu);
 }
 
-template <typename R, int NR, int B, int MASK, int I>
-__device__ __forceinline__ void rotn_fixed(typename C2<R>::T (&x)[NR], const Op& op, const typename C2<R>::T* rcs) {
+template <typename R, int B, int I, bool ALL>
+__device__ __forceinline__ void rotn_bits(Rows<R, B>& x, uint32_t ku, const R (&t)[5]) {
   if constexpr (I < B) {
-    if constexpr (((MASK >> I) & 1) != 0) rot_tan<R, NR, (1 << I)>(x, rcs[rotn_slot(op, I)].x);
-    rotn_fixed<R, NR, B, MASK, I + 1>(x, op, rcs);
+    if (ALL || ((ku >> I) & 1)) rot_tan<(1 << I)>(x, t[I]);
+    rotn_bits<R, B, I + 1, ALL>(x, ku, t);
   }
 }
 
-template <typename R, int NR, int B, int I>
-__device__ __forceinline__ void rotn_any(typename C2<R>::T (&x)[NR], const Op& op, const typename C2<R>::T* rcs) {
-  if constexpr (I < B) {
-    if ((op.ku >> I) & 1) rot_tan<R, NR, (1 << I)>(x, rcs[rotn_slot(op, I)].x);
-    rotn_any<R, NR, B, I + 1>(x, op, rcs);
+template <typename R, int B>
+__device__ __forceinline__ void rotn(Rows<R, B>& x, uint32_t ku, const R (&t)[5]) {
+  constexpr uint32_t kUpper = ((1u << B) - 1u) & ~1u;
+  if (sizeof(R) == 4 && (ku & kUpper) == kUpper) {
+    if (ku & 1u) rot_tan<1>(x, t[0]);
+    rotn_bits<R, B, 1, true>(x, ku, t);
+  } else {
+    rotn_bits<R, B, 0, false>(x, ku, t);
   }
 }
 
-template <typename R, int NR, int B, int I>
-__device__ __forceinline__ void flip_run(typename C2<R>::T (&x)[NR], uint32_t fl) {
+template <typename R, int B, int I>
+__device__ __forceinline__ void flip_run(Rows<R, B>& x, uint32_t fl) {
   if constexpr (I < B) {
-    if ((fl >> I) & 1) flip_pairs<R, NR, (1 << I)>(x);
-    flip_run<R, NR, B, I + 1>(x, fl);
+    if ((fl >> I) & 1) flip_pairs<R, (1 << I)>(x);
+    flip_run<R, B, I + 1>(x, fl);
   }
-}
-
-template <typename R, int NR, int B>
-__device__ __forceinline__ void rot_run(typename C2<R>::T (&x)[NR], const Op& op, const typename C2<R>::T* rcs,
-                                        uint32_t fl) {
-  constexpr int FULL = (1 << B) - 1;
-  if (op.ku == FULL)
-    rotn_fixed<R, NR, B, FULL, 0>(x, op, rcs);
-  else if (op.ku == (FULL & ~1))
-    rotn_fixed<R, NR, B, (FULL & ~1), 0>(x, op, rcs);
-  else
-    rotn_any<R, NR, B, 0>(x, op, rcs);
-  if (fl) flip_run<R, NR, B, 0>(x, fl);
 }
 
 // DROT: x[k] <- (cos - i sin (-1)^popcount(z & r_k)) x[k], the rotation of one
 // diagonal term; sb is the parity of z over the row's fixed bits.
-template <typename R, int NR>
-__device__ __forceinline__ void diag_rot(typename C2<R>::T (&x)[NR], R c, R s, uint32_t zk, int sb) {
+template <typename R, int B>
+__device__ __forceinline__ void diag_rot(Rows<R, B>& x, R c, R s, uint32_t zk, int sb) {
   using T2 = typename C2<R>::T;
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
+  for (int k = 0; k < (1 << B); ++k) {
     const R ss = (sb ^ parity(zk & uint32_t(k))) ? -s : s;
-    const T2 v = x[k];
-    x[k] = T2{fma(ss, v.y, c * v.x), fma(-ss, v.x, c * v.y)};
+    const T2 v = x.get(k);
+    x.set(k, T2{fma(ss, v.y, c * v.x), fma(-ss, v.x, c * v.y)});
   }
 }
 
 // Register flips the planner may emit: one or two register bits.
-#define HS_Q_KU_LIST(X) \
-  X(1) X(2) X(4) X(8) X(16) X(3) X(5) X(6) X(9) X(10) X(12) X(17) X(18) X(20) X(24)
+#define HS_Q_KU2_LIST(X) X(3) X(5) X(6) X(9) X(10) X(12) X(17) X(18) X(20) X(24)
+#define HS_Q_KU_LIST(X) X(1) X(2) X(4) X(8) X(16) HS_Q_KU2_LIST(X)
 
-template <typename R, int NR>
-__device__ __forceinline__ void rot_dispatch(typename C2<R>::T (&x)[NR], int ku, R c, R s, bool fast, int q,
-                                          uint32_t zk, int sb, bool flip) {
+template <typename R, int B>
+__device__ __forceinline__ void rot_dispatch(Rows<R, B>& x, int ku, R c, R s, bool fast, int q, uint32_t zk, int sb,
+                                             bool flip) {
   switch (ku) {
 #define HS_Q_ROT_CASE(K) \
   case K:                \
-    if constexpr (K < NR) rot_ku<R, NR, K>(x, c, s, fast, q, zk, sb, flip); \
+    if constexpr (K < (1 << B)) rot_ku<R, K>(x, c, s, fast, q, zk, sb, flip); \
     break;
     HS_Q_KU_LIST(HS_Q_ROT_CASE)
 #undef HS_Q_ROT_CASE
@@ -266,15 +387,15 @@ __device__ __forceinline__ void rot_dispatch(typename C2<R>::T (&x)[NR], int ku,
   }
 }
 
-template <typename R, int NR>
-__device__ __forceinline__ void tan_dispatch(typename C2<R>::T (&x)[NR], int ku, R t, bool flip) {
+template <typename R, int B>
+__device__ __forceinline__ void tan_dispatch(Rows<R, B>& x, int ku, R t, bool flip) {
   switch (ku) {
-#define HS_Q_TAN_CASE(K)                  \
-  case K:                                 \
-    if constexpr (K < NR) {               \
-      rot_tan<R, NR, K>(x, t);            \
-      if (flip) flip_pairs<R, NR, K>(x);  \
-    }                                     \
+#define HS_Q_TAN_CASE(K)                \
+  case K:                               \
+    if constexpr (K < (1 << B)) {       \
+      rot_tan<K>(x, t);                 \
+      if (flip) flip_pairs<R, K>(x);    \
+    }                                   \
     break;
     HS_Q_KU_LIST(HS_Q_TAN_CASE)
 #undef HS_Q_TAN_CASE
@@ -282,14 +403,27 @@ __device__ __forceinline__ void tan_dispatch(typename C2<R>::T (&x)[NR], int ku,
   }
 }
 
-template <typename R, int NR, int B>
-__device__ __forceinline__ void tab_dispatch(typename C2<R>::T (&x)[NR], int ku, const typename C2<R>::T* tb, int ns,
-                                          uint32_t pt, const uint32_t (&pr)[B]) {
+template <typename R, int B>
+__device__ __forceinline__ void bond_dispatch(Rows<R, B>& x, int ku, typename C2<R>::T w) {
   switch (ku) {
-    case 0: tab_ku<R, NR, B, 0>(x, tb, ns, pt, pr); break;
+#define HS_Q_BOND_CASE(K) \
+  case K:                 \
+    if constexpr (K < (1 << B)) bond_rows<R, K>(x, w); \
+    break;
+    HS_Q_KU2_LIST(HS_Q_BOND_CASE)
+#undef HS_Q_BOND_CASE
+    default: break;
+  }
+}
+
+template <typename R, int B>
+__device__ __forceinline__ void tab_dispatch(Rows<R, B>& x, int ku, const typename C2<R>::T* tb, int ns, uint32_t pt,
+                                             const uint32_t (&pr)[B]) {
+  switch (ku) {
+    case 0: tab_ku<R, B, 0>(x, tb, ns, pt, pr); break;
 #define HS_Q_TAB_CASE(K) \
   case K:                \
-    if constexpr (K < NR) tab_ku<R, NR, B, K>(x, tb, ns, pt, pr); \
+    if constexpr (K < (1 << B)) tab_ku<R, B, K>(x, tb, ns, pt, pr); \
     break;
     HS_Q_KU_LIST(HS_Q_TAB_CASE)
 #undef HS_Q_TAB_CASE
@@ -303,131 +437,240 @@ __device__ __forceinline__ void tab_dispatch(typename C2<R>::T (&x)[NR], int ku,
 // E[mu] = sum over the classes with register part mu of +-C_c, the phase of
 // register row k is e0 * prod_mu exp(-i pi E[mu] chi_mu(k)), chi_mu(k) =
 // (-1)^popcount(mu & k).  The factors of mu = 0 and of the single register
-// bits are multiplied out in two small groups of bits (all rows' values from
-// a few products); every other mu present multiplies each row by
-// cos(pi E) -+ i sin(pi E).  One sincospi per present mu, not per row.
-// ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ R class_sum(const PClass* cls, const R* Cs, int c0, int c1, uint32_t lt) {
-  R e = R(0);
-  for (int cc = c0; cc < c1; ++cc) {
-    const R v = Cs[cc];
-    e += parity(cls[cc].thr & lt) ? -v : v;
-  }
-  return e;
-}
-
-template <typename R, int NR, int B>
-__device__ __forceinline__ void phase_apply(typename C2<R>::T (&x)[NR], const Phase& P, const PClass* cls,
-                                            const R* Cs, typename C2<R>::T e0, uint32_t lt) {
-  using T2 = typename C2<R>::T;
-  constexpr int B1 = (B + 1) / 2, B2 = B - B1;  // the single-bit factors in two groups
-  const int base = P.cls0;
-  // mu = 0 (thread-dependent part of the constant) folded into e0.
-  T2 g0 = e0;
-  {
-    const R e = class_sum<R>(cls, Cs, base + P.mu_beg[0], base + P.mu_beg[1], lt);
-    R sn, cn;
-    sincospi_r(e, &sn, &cn);
-    g0 = T2{fma(g0.x, cn, g0.y * sn), fma(g0.y, cn, -g0.x * sn)};
-  }
-  // Single register bits: (cos, sin) of pi E[2^i].
-  R cb[B], sb[B];
-#pragma unroll
-  for (int i = 0; i < B; ++i) {
-    const int mu = 1 << i;
-    const R e = class_sum<R>(cls, Cs, base + P.mu_beg[mu], base + P.mu_beg[mu + 1], lt);
-    sincospi_r(e, &sb[i], &cb[i]);
-  }
-  // Group values, applied one group at a time (fewer live registers):
-  // A[a] = g0 prod_{i < B1} f_i(bit i of a), then Bv[b] = prod_{i < B2}
-  // f_{B1+i}(bit i of b); f_i(0) = cos - i sin, f_i(1) = cos + i sin.  A
-  // pattern mu of two or more register bits within one group multiplies that
-  // group's values; one that spans both groups multiplies every row.
-  uint32_t rest = P.mu_mask;
-#pragma unroll
-  for (int i = 0; i <= B; ++i) rest &= ~(i == 0 ? 1u : (1u << (1 << (i - 1))));
-  constexpr uint32_t GA = (1u << B1) - 1u;
-  auto mu_factor = [&](int mu, R& cn, R& sn) {
-    const R e = class_sum<R>(cls, Cs, base + P.mu_beg[mu], base + P.mu_beg[mu + 1], lt);
-    sincospi_r(e, &sn, &cn);
-  };
-  {
-    T2 A[1 << B1];
-    A[0] = g0;
-#pragma unroll
-    for (int i = 0; i < B1; ++i)
-#pragma unroll
-      for (int k = 0; k < (1 << i); ++k) {
-        const T2 p = A[k];
-        const R ac = p.x * cb[i], bs = p.y * sb[i], bc = p.y * cb[i], as = p.x * sb[i];
-        A[k] = T2{ac + bs, bc - as};
-        A[k + (1 << i)] = T2{ac - bs, bc + as};
-      }
-    for (uint32_t r = rest & ((1u << (1u << B1)) - 1u); r; r &= r - 1u) {  // mu inside group A
-      const int mu = __ffs(r) - 1;
-      R cn, sn;
-      mu_factor(mu, cn, sn);
-#pragma unroll
-      for (int k = 0; k < (1 << B1); ++k) A[k] = cmul<T2, R>(A[k], cn, parity(uint32_t(mu) & uint32_t(k)) ? sn : -sn);
-    }
-#pragma unroll
-    for (int k = 0; k < NR; ++k) x[k] = cmul<T2, R>(x[k], A[k & GA].x, A[k & GA].y);
-  }
-  {
-    T2 Bv[1 << B2];
-    Bv[0] = T2{R(1), R(0)};
-#pragma unroll
-    for (int i = 0; i < B2; ++i)
-#pragma unroll
-      for (int k = 0; k < (1 << i); ++k) {
-        const T2 p = Bv[k];
-        const R c = cb[B1 + i], sn = sb[B1 + i];
-        const R ac = p.x * c, bs = p.y * sn, bc = p.y * c, as = p.x * sn;
-        Bv[k] = T2{ac + bs, bc - as};
-        Bv[k + (1 << i)] = T2{ac - bs, bc + as};
-      }
-    for (uint32_t r = rest; r; r &= r - 1u) {  // mu inside group B
-      const int mu = __ffs(r) - 1;
-      if (uint32_t(mu) & GA) continue;
-      R cn, sn;
-      mu_factor(mu, cn, sn);
-#pragma unroll
-      for (int k = 0; k < (1 << B2); ++k)
-        Bv[k] = cmul<T2, R>(Bv[k], cn, parity(uint32_t(mu >> B1) & uint32_t(k)) ? sn : -sn);
-    }
-#pragma unroll
-    for (int k = 0; k < NR; ++k) x[k] = cmul<T2, R>(x[k], Bv[k >> B1].x, Bv[k >> B1].y);
-  }
-  for (uint32_t r = rest; r; r &= r - 1u) {  // mu across the two groups
-    const int mu = __ffs(r) - 1;
-    if (!(uint32_t(mu) & GA) || uint32_t(mu) <= GA) continue;
-    R cn, sn;
-    mu_factor(mu, cn, sn);
-#pragma unroll
-    for (int k = 0; k < NR; ++k) {
-      const R ss = parity(uint32_t(mu) & uint32_t(k)) ? sn : -sn;
-      x[k] = cmul<T2, R>(x[k], cn, ss);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The sweep of units [u0, u1) of one descriptor (single launch: the kernel
-// parameter; batched launch: a descriptor in global memory).  NT = 2^(T - B)
-// threads; NR = 2^B rows per thread.
+// bits are multiplied out in two small groups of bits (all rows' values from a
+// few products), with the patterns of two or more bits inside a group; a
+// pattern across the groups multiplies every row.
 //
-// A unit's tile moves HBM -> shared memory -> registers by warp-cooperative
+// A thread's factors go through its own slots of shared memory: slot 0 the
+// product of e0 and mu = 0, slots 1 .. B (cos, sin) of the single register
+// bits, then one (cos, sin) per pattern inside a group and per pattern across
+// the groups, ascending (Args::fac_keep; otherwise those across take turns in
+// one slot).  One sincospi per slot, not per row, in one loop.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void sincospi_r(float x, float* s, float* c) { sincospif(x, s, c); }
+__device__ __forceinline__ void sincospi_r(double x, double* s, double* c) { sincospi(x, s, c); }
+
+template <typename R>
+struct ClassC {
+  R c;           // the class constant of the tile
+  uint32_t thr;  // local part on thread positions
+};
+
+template <typename R>
+__device__ __forceinline__ void phase_factor(const Phase& P, const ClassC<R>* cw, int mu, uint32_t lt, R* sn, R* cn) {
+  R e = R(0);
+  const int c1 = P.cls0 + P.mu_beg[mu + 1];
+#pragma unroll 1
+  for (int cc = P.cls0 + P.mu_beg[mu]; cc < c1; ++cc) {
+    const ClassC<R> C = cw[cc];
+    e += flip_sign(C.c, uint32_t(__popc(C.thr & lt)));
+  }
+  sincospi_r(e, sn, cn);
+}
+
+// A[k], k over N register bits, from A[0] and the bits' (cos, sin): f_i(0) =
+// cos - i sin, f_i(1) = cos + i sin; then the patterns (in coordinates of the
+// N bits) listed in `pats`, from the slots at `f`.
+template <typename T2, typename R, int N>
+__device__ __forceinline__ void group_values(T2 (&A)[1 << N], const T2* cs, uint32_t pats, const T2*& f, int nt) {
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int k = 0; k < (1 << i); ++k) {
+      const T2 p = A[k];
+      const R ac = p.x * cs[i].x, bs = p.y * cs[i].y, bc = p.y * cs[i].x, as = p.x * cs[i].y;
+      A[k] = T2{ac + bs, bc - as};
+      A[k + (1 << i)] = T2{ac - bs, bc + as};
+    }
+#pragma unroll 1
+  for (uint32_t r = pats; r; r &= r - 1u, f += nt) {
+    const int mu = __ffs(r) - 1;
+    const T2 v = *f;
+#pragma unroll
+    for (int k = 0; k < (1 << N); ++k) A[k] = cmul<T2, R>(A[k], v.x, parity(uint32_t(mu) & uint32_t(k)) ? v.y : -v.y);
+  }
+}
+
+// Register bits 0 .. B1 - 1 form the lower group, the others the upper one.
+__host__ __device__ constexpr int lower_bits(int B) { return (B + 1) / 2; }
+
+template <int B>
+__device__ __forceinline__ void phase_apply(Rows<float, B>& x, uint32_t mu_mask, const float2* fac, int nt) {
+  constexpr int B1 = lower_bits(B), B2 = B - B1;
+  float2 cs[B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) cs[i] = fac[(1 + i) * nt];
+  const float2* f = fac + (1 + B) * nt;
+  {
+    float2 A[1 << B1];
+    A[0] = fac[0];
+    group_values<float2, float, B1>(A, cs, lower_patterns<B>(mu_mask), f, nt);
+#pragma unroll
+    for (int a = 0; a < (1 << (B1 - 1)); ++a) {
+      const float2 c = make_float2(A[2 * a].x, A[2 * a + 1].x), s = make_float2(A[2 * a].y, A[2 * a + 1].y), ns = neg2(s);
+#pragma unroll
+      for (int b = 0; b < (1 << B2); ++b) {
+        const int j = a + (b << (B1 - 1));
+        const float2 r = x.re[j], m = x.im[j];
+        x.re[j] = fma2(r, c, __fmul2_rn(m, ns));
+        x.im[j] = fma2(r, s, __fmul2_rn(m, c));
+      }
+    }
+  }
+  {
+    float2 A[1 << B2];
+    A[0] = make_float2(1.0f, 0.0f);
+    group_values<float2, float, B2>(A, cs + B1, upper_patterns<B>(mu_mask), f, nt);
+#pragma unroll
+    for (int b = 0; b < (1 << B2); ++b) {
+      const float2 c = dup(A[b].x), s = dup(A[b].y), ns = dup(-A[b].y);
+#pragma unroll
+      for (int a = 0; a < (1 << (B1 - 1)); ++a) {
+        const int j = a + (b << (B1 - 1));
+        const float2 r = x.re[j], m = x.im[j];
+        x.re[j] = fma2(r, c, __fmul2_rn(m, ns));
+        x.im[j] = fma2(r, s, __fmul2_rn(m, c));
+      }
+    }
+  }
+}
+
+template <int B>
+__device__ __forceinline__ void pattern_apply(Rows<float, B>& x, int mu, float2 v) {
+  constexpr int NP = 1 << (B - 1);
+  const float2 c = dup(v.x);
+  // row 2j + h takes cos - i sin (-1)^popcount(mu & (2j + h))
+  const float2 s0 = make_float2(v.y, flip_sign(v.y, uint32_t(mu)));
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    const uint32_t sg = uint32_t(__popc(mu & (2 * j)));
+    const float2 s = make_float2(flip_sign(s0.x, sg), flip_sign(s0.y, sg)), ns = neg2(s);
+    const float2 r = x.re[j], m = x.im[j];
+    x.re[j] = fma2(r, c, __fmul2_rn(m, s));
+    x.im[j] = fma2(r, ns, __fmul2_rn(m, c));
+  }
+}
+
+template <int B>
+__device__ __forceinline__ void phase_apply(Rows<double, B>& x, uint32_t mu_mask, const double2* fac, int nt) {
+  constexpr int B1 = lower_bits(B), B2 = B - B1;
+  double2 cs[B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) cs[i] = fac[(1 + i) * nt];
+  const double2* f = fac + (1 + B) * nt;
+  double2 A[1 << B1], C[1 << B2];
+  A[0] = fac[0];
+  group_values<double2, double, B1>(A, cs, lower_patterns<B>(mu_mask), f, nt);
+  C[0] = make_double2(1.0, 0.0);
+  group_values<double2, double, B2>(C, cs + B1, upper_patterns<B>(mu_mask), f, nt);
+#pragma unroll
+  for (int k = 0; k < (1 << B); ++k) x.x[k] = cmul<double2, double>(x.x[k], A[k & ((1 << B1) - 1)].x, A[k & ((1 << B1) - 1)].y);
+#pragma unroll
+  for (int k = 0; k < (1 << B); ++k) x.x[k] = cmul<double2, double>(x.x[k], C[k >> B1].x, C[k >> B1].y);
+}
+
+template <int B>
+__device__ __forceinline__ void pattern_apply(Rows<double, B>& x, int mu, double2 v) {
+#pragma unroll
+  for (int k = 0; k < (1 << B); ++k) x.x[k] = cmul<double2, double>(x.x[k], v.x, parity(mu & k) ? v.y : -v.y);
+}
+
+// The whole op; `fresh`: the factors are not in the slots yet.
+template <typename R, int B>
+__device__ __forceinline__ void phase_op(Rows<R, B>& x, const Phase& P, const ClassC<R>* cw, typename C2<R>::T e0,
+                                         uint32_t lt, typename C2<R>::T* fac, int nt, bool fresh, bool keep) {
+  using T2 = typename C2<R>::T;
+  const uint32_t mu_mask = P.mu_mask;
+  // Patterns in the order of their slots: inside the groups, then across.
+  uint32_t inside = inside_patterns<B>(mu_mask), across = across_patterns<B>(mu_mask);
+  const int n_in = B + __popc(inside);  // last slot of the first round
+  int slot = 0, last = n_in, mu = 0;
+#pragma unroll 1
+  while (true) {
+    if (fresh) {
+#pragma unroll 1
+      for (int k = slot; k <= last; ++k) {
+        if (k <= B) {
+          mu = k == 0 ? 0 : 1 << (k - 1);
+        } else if (k <= n_in) {
+          mu = __ffs(inside) - 1;
+          inside &= inside - 1u;
+        }
+        R sn, cn;
+        phase_factor<R>(P, cw, mu, lt, &sn, &cn);
+        fac[k * nt] = mu == 0 ? cmul<T2, R>(e0, cn, -sn) : T2{cn, sn};
+      }
+    }
+    if (slot == 0)
+      phase_apply<B>(x, mu_mask, fac, nt);
+    else
+      pattern_apply<B>(x, mu, fac[slot * nt]);
+    if (!across) break;
+    mu = __ffs(across) - 1;
+    across &= across - 1u;
+    slot = (slot == 0 || !keep) ? n_in + 1 : slot + 1;
+    last = slot;
+  }
+}
+
+// Byte offsets of a CTA's tables in shared memory (the tile comes first).
+struct SmemMap {
+  uint32_t ops, lays, fac, vts, e0s, cw, ph, cls, pt, thpi, clane, scale, total;
+};
+
+// An op with its coefficients; a layout with the local row (x) and the
+// swizzled chunk (y) that a lane index (0 .. 31) and a warp index (32 ..)
+// deposit: a thread's register row 0 is the XOR of the two.
+template <typename R>
+struct OpRec {
+  Op op;
+  Coef<R> c;
+};
+struct LayRec {
+  Layout L;
+  uint2 dep[48];
+};
+
+__host__ __device__ __forceinline__ SmemMap smem_map(const Args& a, uint32_t e, uint32_t nt) {
+  SmemMap m;
+  uint32_t o = e << a.tile_bits;
+  auto take = [&](uint32_t bytes) {
+    const uint32_t at = o;
+    o += (bytes + 15u) & ~15u;
+    return at;
+  };
+  const uint32_t warps = nt >> 5;
+  m.ops = take((e == 8 ? sizeof(OpRec<float>) : sizeof(OpRec<double>)) * a.n_ops);
+  m.lays = take(sizeof(LayRec) * a.n_lay);
+  m.fac = take(e * nt * a.n_fac);
+  m.vts = take(e * a.n_vt);
+  m.e0s = take(e * warps * a.n_phase);
+  m.cw = take(e * warps * a.n_cls);  // sizeof(ClassC<R>) = the element size
+  m.ph = take(sizeof(Phase) * a.n_phase);
+  m.cls = take(sizeof(PClass) * a.n_cls);
+  m.pt = take(sizeof(PTerm) * a.n_pterm);
+  m.thpi = take((e / 2) * a.n_pterm);
+  m.clane = take(48 * 4);
+  m.scale = take(e);
+  m.total = o;
+  return m;
+}
+
+// ---------------------------------------------------------------------------
+// The sweep of chunks q0, q0 + stride, ... < q1 of one descriptor (single
+// launch: the kernel parameter; batched launch: a descriptor in global
+// memory).  NT = 2^(T - B) threads; NR = 2^B rows per thread.
+//
+// A state's tile moves HBM -> shared memory -> registers by warp-cooperative
 // copies (each warp copies exactly the rows its threads hold in the first
 // layout, in address order), so the first read needs only a warp barrier.
-// Once a unit has read its last layout, the tile buffer is free: after one CTA
-// barrier every warp starts copying its rows of the CTA's next unit, which
-// land while the current unit finishes in registers and writes its rows
-// straight back to HBM.
+// Once its last layout has been read, the tile buffer is free: every warp
+// starts copying its rows of the CTA's next state or tile, which land while
+// the current one finishes in registers and goes straight back to HBM.
 // ---------------------------------------------------------------------------
 template <typename R, int B, bool FULL>
-__device__ __forceinline__ void qsweep_core(const Args& a, uint32_t u0, uint32_t u1, unsigned char* smem_raw,
-                                            bool pdl) {
+__device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t q1, uint32_t stride,
+                                            unsigned char* smem_raw, bool pdl) {
   using T2 = typename C2<R>::T;
   constexpr int NR = 1 << B;
   constexpr int V = 16 / int(sizeof(T2));  // rows per 16-byte chunk (2 for complex64)
@@ -435,42 +678,16 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t u0, uint32_t
   constexpr int NJ = NR / V;               // chunks per thread
   const int NT = blockDim.x;
   const uint32_t tid = threadIdx.x;
-  const uint32_t TS = 1u << a.tile_bits;
   const uint32_t m0 = a.m0, m1 = a.m1;
   const int sh = a.sh;
-  const int n_warps = NT >> 5;
   const int warp = tid >> 5, lane = tid & 31;
 
-  // Shared memory: [tile][value tables][rotations][per-warp e0 per phase]
-  // [per-warp class constants][ops][layouts][phase headers][classes][terms]
-  // [term angles][scale partials]
+  const SmemMap sm = smem_map(a, sizeof(T2), NT);
+  auto at = [&](uint32_t SmemMap::* field) -> unsigned char* { return smem_raw + sm.*field; };
   T2* tile = reinterpret_cast<T2*>(smem_raw);
-  T2* vts = tile + TS;  // 16-byte aligned (the planner keeps n_vt and every table start even)
-  T2* rcs = vts + a.n_vt;
-  T2* e0s = rcs + a.n_rot + warp * a.n_phase;
-  R* Cs = reinterpret_cast<R*>(rcs + a.n_rot + n_warps * a.n_phase) + warp * a.n_cls;
-  unsigned char* meta = reinterpret_cast<unsigned char*>(
-      reinterpret_cast<R*>(rcs + a.n_rot + n_warps * a.n_phase) + n_warps * a.n_cls);
-  meta += (16 - reinterpret_cast<uintptr_t>(meta) % 16) % 16;
-  Op* sops = reinterpret_cast<Op*>(meta);
-  Layout* slay = reinterpret_cast<Layout*>(sops + a.n_ops);
-  Phase* sph = reinterpret_cast<Phase*>(slay + a.n_lay);
-  PClass* scls = reinterpret_cast<PClass*>(sph + a.n_phase);
-  PTerm* spt = reinterpret_cast<PTerm*>(scls + a.n_cls);
-  auto align16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15); };
-  R* thpi = reinterpret_cast<R*>(align16(spt + a.n_pterm));
-  double* mpart = reinterpret_cast<double*>(align16(thpi + a.n_pterm));
-  int* kpart = reinterpret_cast<int*>(mpart + n_warps);
-  uint8_t* flips = reinterpret_cast<uint8_t*>(kpart + n_warps);  // per op: register bits whose partners swap
-  // Per layout: the local-row bits a lane index and a warp index deposit
-  // (local row of a thread's register row 0 = dlane[lane] | dwarp[warp]).
-  uint32_t* dlane = reinterpret_cast<uint32_t*>(align16(flips + a.n_ops));
-  uint32_t* dwarp = dlane + 32 * a.n_lay;
-
-  auto unit_base = [&](uint32_t unit) { return deposit_runs(unit & ((1u << a.n_tiles_log2) - 1u), a.rest); };
-  auto unit_src = [&](uint32_t unit) {
-    return reinterpret_cast<const T2*>(a.src) + HS_BCHK(unit >> a.n_tiles_log2, a.n_rhs, BS_REG_STATE) * a.N;
-  };
+  OpRec<R>* ops = reinterpret_cast<OpRec<R>*>(smem_raw + sm.ops);
+  LayRec* lays = reinterpret_cast<LayRec*>(smem_raw + sm.lays);
+  T2* fac = reinterpret_cast<T2*>(smem_raw + sm.fac) + tid;
 
   // Per-CTA tables (written by launches that completed before this grid began).
   {
@@ -479,113 +696,120 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t u0, uint32_t
       uint32_t* d4 = static_cast<uint32_t*>(dst);
       for (uint32_t w = tid; w < bytes / 4; w += NT) d4[w] = s4[w];
     };
-    copy_words(sops, a.ops, sizeof(Op) * a.n_ops);
-    copy_words(slay, a.lay, sizeof(Layout) * a.n_lay);
-    copy_words(sph, a.ph, sizeof(Phase) * a.n_phase);
-    copy_words(scls, a.cls, sizeof(PClass) * a.n_cls);
-    copy_words(spt, a.pt, sizeof(PTerm) * a.n_pterm);
+    for (int i = 0; i < a.n_lay; ++i) copy_words(&lays[i].L, a.lay + i, sizeof(Layout));
+    copy_words(smem_raw + sm.ph, a.ph, sizeof(Phase) * a.n_phase);
+    copy_words(smem_raw + sm.cls, a.cls, sizeof(PClass) * a.n_cls);
+    copy_words(smem_raw + sm.pt, a.pt, sizeof(PTerm) * a.n_pterm);
   }
   for (int e = tid; e < 48 * a.n_lay; e += NT) {
     const int li = e / 48, j = e - 48 * li;
     const Layout& L = a.lay[li];
     uint32_t d = 0;
-    if (j < 32) {
+    if (j < 32)
       for (int i = 0; i < 5 && i < L.n_thr; ++i) d |= uint32_t((j >> i) & 1) << L.thr[i];
-      dlane[32 * li + j] = d;
+    else
+      for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
+    lays[li].dep[j] = make_uint2(d, swz(d >> VB));
+  }
+  // The local rows that a lane and a warp index deposit in the copies of the
+  // first layout's rows in address order.
+  uint32_t* clane_s = reinterpret_cast<uint32_t*>(smem_raw + sm.clane);
+  for (int j = tid; j < 48; j += NT) {
+    const Layout& L = a.lay[a.ops[0].idx];
+    uint32_t d = 0;
+    if (j < 32) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) d |= uint32_t((j >> k) & 1) << (L.wlo[k] + VB);
     } else {
       for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
-      dwarp[16 * li + (j - 32)] = d;
     }
+    clane_s[j] = d;
   }
-  // Rotations: a fast rotation (y = 0, z = 0) as tan(theta') of the factor
-  // build's record, with cos(theta') and its quarter turns k in the sweep's
-  // scale (the warps' partial products and sums, combined where the scale is
-  // applied) and an odd k as a swap of partners in its op; any other rotation
-  // as (cos, sin).
-  for (int i = tid; i < a.n_rot; i += NT) {
-    const int e = a.rot[i].cs;
-    if (a.rot[i].fast) {
-      const double* q = a.rq + 4 * HS_BCHK(e, a.n_terms_g, BS_REG_TERM);
-      rcs[i] = T2{R(q[0]), R(0)};
-    } else {
-      const double* p = a.cs + 2 * HS_BCHK(e, a.n_terms_g, BS_REG_TERM);
-      rcs[i] = T2{R(p[0]), R(p[1])};
-    }
-  }
-  {
-    double m = 1.0;
-    int kq = 0;
-    auto take = [&](int rot) {
-      const double* q = a.rq + 4 * HS_BCHK(a.rot[rot].cs, a.n_terms_g, BS_REG_TERM);
-      m *= q[2];
-      const int k = int(q[1]);
-      kq += k;
-      return k & 1;
-    };
-    for (int oi = tid; oi < a.n_ops; oi += NT) {
-      const Op& op = a.ops[oi];
-      uint32_t fl = 0;
-      if (op.type == OP_ROT && (op.flags & 1)) {
-        fl = uint32_t(take(op.idx));
-      } else if (op.type == OP_ROTN) {
-#pragma unroll
-        for (int i = 0; i < B; ++i)
-          if ((op.ku >> i) & 1) fl |= uint32_t(take(rotn_slot(op, i))) << i;
-      }
-      flips[oi] = uint8_t(fl);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      m *= __shfl_xor_sync(0xffffffffu, m, o);
-      kq += __shfl_xor_sync(0xffffffffu, kq, o);
-    }
-    if (lane == 0) {
-      mpart[warp] = m;
-      kpart[warp] = kq;
-    }
-  }
-  for (int t = tid; t < a.n_pterm; t += NT) thpi[t] = R(a.rq[4 * HS_BCHK(a.pt[t].th, a.n_terms_g, BS_REG_TERM) + 3]);
+  R* thpi_s = reinterpret_cast<R*>(smem_raw + sm.thpi);
+  for (int t = tid; t < a.n_pterm; t += NT) thpi_s[t] = R(a.rq[4 * HS_BCHK(a.pt[t].th, a.n_terms_g, BS_REG_TERM) + 3]);
+  T2* vts = reinterpret_cast<T2*>(smem_raw + sm.vts);
   for (int t = 0; t < a.n_tab; ++t) {
     const T2* g = reinterpret_cast<const T2*>(a.vt) + a.tab[t].vt0;
     const int s0 = a.tab[t].s0, n = a.tab[t].n;
     for (int e = tid; e < n; e += NT) vts[s0 + e] = g[HS_BCHK(a.tab[t].vt0 + e, a.n_vt_g, BS_REG_VT) - a.tab[t].vt0];
   }
+  // Coefficients of every op, and the sweep's scale (the same for every tile):
+  // the product of the fast rotations' cos(theta') and quarter turns (-i)^k
+  // and of the bonds' phases e^{-i theta}.  One warp does this, in FP64: the
+  // FP64 pipe takes tens of cycles per warp instruction, so the others stay
+  // off it.
+  if (warp == 0) {
+    double m = 1.0, ph = 0.0;
+    int kq = 0;
+    // A fast rotation (y = 0, z = 0): tan(theta') of the factor build's record.
+    auto take = [&](int rot, R& t) {
+      const double* q = a.rq + 4 * HS_BCHK(a.rot[rot].cs, a.n_terms_g, BS_REG_TERM);
+      t = R(q[0]);
+      m *= q[2];
+      const int k = int(q[1]);
+      kq += k;
+      return uint32_t(k & 1);
+    };
+    for (int oi = lane; oi < a.n_ops; oi += 32) {
+      const Op& op = a.ops[oi];
+      Coef<R> c;
+      c.swap = 0;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) c.v[i] = R(0);
+      if (op.type == OP_ROTN) {
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+          if ((op.ku >> i) & 1) c.swap |= take(rotn_slot(op, i), c.v[i]) << i;
+      } else if (op.type == OP_ROT && (op.flags & 1)) {
+        c.swap = take(op.idx, c.v[0]);
+      } else if (op.type == OP_ROT || op.type == OP_DROT) {
+        const double* p = a.cs + 2 * HS_BCHK(a.rot[op.idx].cs, a.n_terms_g, BS_REG_TERM);
+        c.v[0] = R(p[0]);
+        c.v[1] = R(p[1]);
+      } else if (op.type == OP_BOND) {
+        // w = (1 - e^{4 i theta}) / 2 = sin(2 theta) (sin(2 theta) - i cos(2 theta))
+        const int64_t e = HS_BCHK(a.bond[op.idx], a.n_terms_g, BS_REG_TERM);
+        const double cs = a.cs[2 * e], sn = a.cs[2 * e + 1];
+        const double s2 = 2.0 * cs * sn, c2 = fma(-2.0 * sn, sn, 1.0);
+        c.v[0] = R(s2 * s2);
+        c.v[1] = R(-s2 * c2);
+        ph += a.rq[4 * e + 3];  // theta / pi
+      }
+      ops[oi].op = op;
+      ops[oi].c = c;
+    }
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      m *= __shfl_xor_sync(0xffffffffu, m, o);
+      ph += __shfl_xor_sync(0xffffffffu, ph, o);
+      kq += __shfl_xor_sync(0xffffffffu, kq, o);
+    }
+    if (lane == 0) {
+      const double u0 = ph + 0.5 * double(kq & 3), u = u0 - 2.0 * rint(0.5 * u0);
+      double sn, cn;
+      sincospi(u, &sn, &cn);
+      *reinterpret_cast<T2*>(smem_raw + sm.scale) = T2{R(m * cn), R(-m * sn)};
+    }
+  }
   const int n_ops = a.n_ops, n_cls = a.n_cls;
+  const int last_lay = a.last_lay;
 
-  // Index of the last layout op (the tile buffer is free after its reads).
-  int last_lay = 0;
-  for (int oi = 0; oi < n_ops; ++oi)
-    if (a.ops[oi].type == OP_LAYOUT) last_lay = oi;
-
-  // Warp-cooperative copy of this warp's rows of a unit in the first layout of
+  // Warp-cooperative copy of this warp's rows of a tile in the first layout of
   // the sweep into the tile buffer: chunk mm of the thread lies at swizzled
   // chunk s0 ^ mswz(mm) and global row g0 ^ mglob(mm), both maps linear over
   // XOR, so four basis values each give all of them.
   constexpr int NJB = B - VB;  // log2 NJ
-  uint32_t cin_s0, cin_g0;
-  {
-    const Layout& L = a.lay[a.ops[0].idx];
-    uint32_t lc = 0;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) lc |= uint32_t((lane >> k) & 1) << L.wlo[k];
-    uint32_t wb = 0;
-    for (int i = 5; i < L.n_thr; ++i) wb |= ((tid >> i) & 1u) << L.thr[i];
-    const uint32_t c0 = lc | (wb >> VB);
-    cin_s0 = swz(c0);
-    cin_g0 = global_of(c0 * V, m0, m1, sh);
-  }
-  const Layout* L0 = slay + a.ops[0].idx;  // the first op is always a layout
-  auto copy_in = [&](uint32_t base, const T2* src) {
-    uint32_t ms[NJB], mg[NJB];
-#pragma unroll
-    for (int k = 0; k < NJB; ++k) {
-      ms[k] = L0->mswz[1 << k];
-      mg[k] = L0->mglob[1 << k];
-    }
-    const uint32_t g0 = cin_g0 | base;
+  const Layout* L0 = &lays[a.ops[0].idx].L;  // the first op is always a layout
+  auto copy_in = [&](uint32_t base, int state) {
+    const T2* src = reinterpret_cast<const T2*>(a.src) + HS_BCHK(state, a.n_rhs, BS_REG_STATE) * a.N;
+    const uint4 ms4 = *reinterpret_cast<const uint4*>(L0->mswz), mg4 = *reinterpret_cast<const uint4*>(L0->mglob);
+    const uint32_t ms[4] = {ms4.x, ms4.y, ms4.z, ms4.w}, mg[4] = {mg4.x, mg4.y, mg4.z, mg4.w};
+    const uint32_t* clane = reinterpret_cast<const uint32_t*>(at(&SmemMap::clane));
+    const uint32_t l0 = clane[lane] | clane[32 + warp];
+    const uint32_t s0 = swz(l0 >> VB), g0 = global_of(l0, m0, m1, sh) | base;
 #pragma unroll
     for (int mm = 0; mm < NJ; ++mm) {
-      uint32_t sx = cin_s0, gx = g0;
+      uint32_t sx = s0, gx = g0;
 #pragma unroll
       for (int k = 0; k < NJB; ++k)
         if ((mm >> k) & 1) {
@@ -599,217 +823,276 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t u0, uint32_t
 
   if (pdl) grid_dependency_wait();  // the state written by the previous launch is visible after this
   __syncthreads();                  // the tables are in shared memory
-  if (u0 < u1) copy_in(unit_base(u0), unit_src(u0));
-  // The sweep's rotation scale m (-i)^K (the same for every unit).
-  R m_sweep;
-  int k_sweep;
-  {
-    double md = 1.0;
-    int kq = 0;
-    for (int w = 0; w < n_warps; ++w) {
-      md *= mpart[w];
-      kq += kpart[w];
-    }
-    m_sweep = R(md);
-    k_sweep = kq & 3;
-  }
+
+  // Chunk q: tile index and its states [state, state_end).
+  uint32_t q = q0, base = 0;
+  int state = 0, state_end = 0;
+  auto chunk = [&](uint32_t c, uint32_t& b, int& s0, int& s1) {
+    const uint32_t t = c / uint32_t(a.rhs_chunks);
+    b = deposit_runs(t, a.rest);
+    s0 = int(c - t * uint32_t(a.rhs_chunks)) * a.rhs_chunk;
+    s1 = min(s0 + a.rhs_chunk, a.n_rhs);
+  };
+  chunk(q, base, state, state_end);
+  copy_in(base, state);
   if (pdl) grid_launch_dependents();  // the next sweep may load its tables meanwhile
 
-  for (uint32_t unit = u0; unit < u1; ++unit) {
-    const uint32_t base = unit_base(unit);
-    T2* dst = reinterpret_cast<T2*>(a.dst) + HS_BCHK(unit >> a.n_tiles_log2, a.n_rhs, BS_REG_STATE) * a.N;
+  bool new_tile = true;
+  uint32_t have = 0;  // PHASE runs whose factors are in shared memory for this tile
+  while (true) {
     // Per-tile phase constants, in this warp's copy: class sums of +-theta_j
     // (units of pi, each term reduced mod 2 in FP64 by the factor build) with
     // the signs of the tile's fixed bits, reduced mod 2 again; a constant class
     // becomes its phase op's e0.  (The warp barrier keeps a lane from writing
-    // them while another lane still reads the previous unit's.)
-    __syncwarp();
-    for (int cc = lane; cc < n_cls; cc += 32) {
-      const PClass C = scls[cc];
-      R acc = R(0);
-      for (int t = C.t0; t < C.t0 + C.nt; ++t) {
-        const R v = thpi[t];
-        acc += parity(spt[t].rest & base) ? -v : v;
+    // them while another lane still reads the previous tile's.)
+    if (new_tile) {
+      have = 0;
+      const PClass* scls = reinterpret_cast<const PClass*>(at(&SmemMap::cls));
+      const PTerm* spt = reinterpret_cast<const PTerm*>(at(&SmemMap::pt));
+      const R* thpi = reinterpret_cast<const R*>(at(&SmemMap::thpi));
+      T2* e0s = reinterpret_cast<T2*>(at(&SmemMap::e0s)) + warp * a.n_phase;
+      ClassC<R>* cw = reinterpret_cast<ClassC<R>*>(at(&SmemMap::cw)) + warp * n_cls;
+      __syncwarp();
+      for (int cc = lane; cc < n_cls; cc += 32) {
+        const PClass C = scls[cc];
+        R acc = R(0);
+        for (int t = C.t0; t < C.t0 + C.nt; ++t) acc += flip_sign(thpi[t], uint32_t(__popc(spt[t].rest & base)));
+        const R ur = acc - R(2) * rint(R(0.5) * acc);
+        if (C.c0p >= 0) {
+          R sn, cn;
+          sincospi_r(ur, &sn, &cn);
+          e0s[C.c0p] = T2{cn, -sn};
+          cw[cc].c = R(0);
+        } else {
+          cw[cc].c = ur;
+        }
+        cw[cc].thr = C.thr;
       }
-      const R ur = acc - R(2) * rint(R(0.5) * acc);
-      if (C.c0p >= 0) {
-        R sn, cn;
-        sincospi_r(ur, &sn, &cn);
-        e0s[C.c0p] = T2{cn, -sn};
-        Cs[cc] = R(0);
+      __syncwarp();
+    }
+
+    const int cur_state = state;
+    const uint32_t cur_base = base;
+    // What this CTA runs next.
+    bool more;
+    {
+      if (state + 1 < state_end) {
+        ++state;
+        more = true;
+        new_tile = false;
       } else {
-        Cs[cc] = ur;
+        more = q1 - q > stride;
+        if (more) {
+          q += stride;
+          chunk(q, base, state, state_end);
+        }
+        new_tile = true;
       }
     }
 
-    __syncwarp();
-    T2 x[NR];
-    uint32_t lt = 0, st = 0, gt = 0;  // row of register index 0: local, swizzled chunk, global
-    const Layout* cur = nullptr;      // the register layout in effect
-
+    Rows<R, B> x;
+    int cur = -1;  // the register layout in effect
+    // Local row of this thread's register row 0 in that layout.
+    auto local_row = [&]() { return lays[cur].dep[lane].x | lays[cur].dep[32 + warp].x; };
+    // Its chunk j in the tile buffer: st ^ XOR of qo over the set bits of j.
+    auto chunk_of = [&](uint32_t& st, uint32_t (&qo)[4]) {
+      st = lays[cur].dep[lane].y ^ lays[cur].dep[32 + warp].y;
+      const uint4 v = *reinterpret_cast<const uint4*>(lays[cur].L.qoff);
+      qo[0] = v.x;
+      qo[1] = v.y;
+      qo[2] = v.z;
+      qo[3] = v.w;
+    };
     for (int oi = 0; oi < n_ops; ++oi) {
-      const Op op = sops[oi];
+      const Op op = ops[oi].op;
       if (op.type == OP_LAYOUT) {
-        // A thread writes back only rows of its own warp (each warp owns the
-        // rows with its warp-bit values), so a warp barrier orders those writes
-        // after the warp's reads of the previous layout; the new layout reads
-        // other warps' rows unless its warp bits are the previous ones (flag).
-        if (cur) {
-          __syncwarp();
-          uint32_t q[B];
-#pragma unroll
-          for (int i = 0; i < B; ++i) q[i] = cur->qoff[i];
+        uint32_t st, qo[4];
+        // A thread writes back exactly the rows it read in the layout so far;
+        // the new layout reads rows of its own warp only (flag 1: the warp bits
+        // are the previous layout's) or of all warps.
+        if (cur >= 0) {
+          chunk_of(st, qo);
 #pragma unroll
           for (int j = 0; j < NJ; ++j) {
             uint32_t pc = st;
 #pragma unroll
-            for (int i = 0; i < B - VB; ++i)
-              if ((j >> i) & 1) pc ^= q[i + VB];
-            if constexpr (V == 2) {
-              *reinterpret_cast<float4*>(tile + pc * 2) =
-                  make_float4(x[2 * j].x, x[2 * j].y, x[2 * j + 1].x, x[2 * j + 1].y);
-            } else {
-              tile[pc] = x[j];
-            }
+            for (int i = 0; i < NJB; ++i)
+              if ((j >> i) & 1) pc ^= qo[i];
+            if constexpr (V == 2)
+              *reinterpret_cast<float4*>(tile + pc * 2) = make_float4(x.re[j].x, x.re[j].y, x.im[j].x, x.im[j].y);
+            else
+              tile[pc] = x.x[j];
           }
           if (op.flags & 1)
             __syncwarp();
           else
             __syncthreads();
         } else {
-          cp_async_wait(0);  // this unit's rows, copied by this warp
+          cp_async_wait(0);  // this tile's rows, copied by this warp
           __syncwarp();
         }
-        const Layout* L = slay + op.idx;
-        const uint32_t l = dlane[32 * op.idx + lane] | dwarp[16 * op.idx + warp];
-        uint32_t q[B];
-#pragma unroll
-        for (int i = 0; i < B; ++i) q[i] = L->qoff[i];
-        lt = l;
-        st = swz(l >> VB);
-        gt = global_of(l, m0, m1, sh) | base;
-        cur = L;
+        const bool first = cur < 0;
+        cur = op.idx;
+        chunk_of(st, qo);
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
           uint32_t pc = st;
 #pragma unroll
-          for (int i = 0; i < B - VB; ++i)
-            if ((j >> i) & 1) pc ^= q[i + VB];
+          for (int i = 0; i < NJB; ++i)
+            if ((j >> i) & 1) pc ^= qo[i];
           if constexpr (V == 2) {
             const float4 w = *reinterpret_cast<const float4*>(tile + pc * 2);
-            x[2 * j] = T2{w.x, w.y};
-            x[2 * j + 1] = T2{w.z, w.w};
+            x.re[j] = make_float2(w.x, w.y);
+            x.im[j] = make_float2(w.z, w.w);
           } else {
-            x[j] = tile[pc];
+            x.x[j] = tile[pc];
           }
         }
-        if (oi == last_lay && unit + 1 < u1) {
-          // The tile buffer is free once every warp has read its rows: start
-          // copying the next unit's rows.
-          __syncthreads();
-          copy_in(unit_base(unit + 1), unit_src(unit + 1));
+        if constexpr (V == 2) {
+          // The copied tile holds (re, im) row by row, a written-back one pairs.
+          if (first) {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+              const float t = x.re[j].y;
+              x.re[j].y = x.im[j].x;
+              x.im[j].x = t;
+            }
+          }
+        }
+        if (oi == last_lay && more) {
+          // The tile buffer is free once every warp (the warp itself where it
+          // copies the rows it has just read) has read its rows.
+          if (a.free_local)
+            __syncwarp();
+          else
+            __syncthreads();
+          copy_in(base, state);
         }
       } else if (op.type == OP_ROTN) {
-        rot_run<R, NR, B>(x, op, rcs, flips[oi]);
+        const Coef<R> c = ops[oi].c;
+        rotn<R, B>(x, op.ku, c.v);
+        if (c.swap) flip_run<R, B, 0>(x, c.swap);
+      } else if (op.type == OP_PHASE) {
+        const Phase& P = reinterpret_cast<const Phase*>(at(&SmemMap::ph))[op.idx];
+        const ClassC<R>* cw = reinterpret_cast<const ClassC<R>*>(at(&SmemMap::cw)) + warp * n_cls;
+        const T2 e0 = reinterpret_cast<const T2*>(at(&SmemMap::e0s))[warp * a.n_phase + op.idx];
+        phase_op<R, B>(x, P, cw, e0, local_row(), fac + P.fac0 * NT, NT, !((have >> op.idx) & 1u), a.fac_keep != 0);
+        if (a.fac_keep) have |= 1u << op.idx;
+      } else if (op.type == OP_BOND) {
+        bond_dispatch<R, B>(x, op.ku, T2{ops[oi].c.v[0], ops[oi].c.v[1]});
       } else if (op.type == OP_ROT) {
-        const T2 cs = rcs[op.idx];
+        const R c = ops[oi].c.v[0];
+        const bool swap = ops[oi].c.swap != 0;
         if constexpr (FULL) {
           const bool fast = op.flags & 1;
-          const int sbit = fast ? 0 : (parity(op.zrest & base) ^ parity(op.zthr & lt));
-          rot_dispatch<R, NR>(x, op.ku, cs.x, cs.y, fast, (op.flags >> 1) & 3, op.zk, sbit, flips[oi] != 0);
+          const int sbit = fast ? 0 : (parity(op.zrest & cur_base) ^ parity(op.zthr & local_row()));
+          rot_dispatch<R, B>(x, op.ku, c, ops[oi].c.v[1], fast, (op.flags >> 1) & 3, op.zk, sbit, swap);
         } else {
-          tan_dispatch<R, NR>(x, op.ku, cs.x, flips[oi] != 0);  // the planner sends only tan-form rotations here
+          tan_dispatch<R, B>(x, op.ku, c, swap);  // the planner sends only tan-form rotations here
         }
       } else if (op.type == OP_DROT) {
-        const T2 cs = rcs[op.idx];
-        diag_rot<R, NR>(x, cs.x, cs.y, op.zk, parity(op.zrest & base) ^ parity(op.zthr & lt));
-      } else if (op.type == OP_TAB) {
+        diag_rot<R, B>(x, ops[oi].c.v[0], ops[oi].c.v[1], op.zk, parity(op.zrest & cur_base) ^ parity(op.zthr & local_row()));
+      } else {
         if constexpr (FULL) {
           const Tab& tb = a.tab[op.idx];
-          const uint32_t sm = tb.sm;
+          const uint32_t smask = tb.sm;
           const int tsh = tb.sh;
           uint32_t pr[B];
 #pragma unroll
-          for (int i = 0; i < B; ++i) pr[i] = pattern_fast(cur->goff[i], sm, tsh);
-          tab_dispatch<R, NR, B>(x, op.ku, vts + tb.s0, tb.ns, pattern_fast(gt, sm, tsh), pr);
+          for (int i = 0; i < B; ++i)
+            pr[i] = pattern_fast(i < VB ? lays[cur].L.g0 : lays[cur].L.goff[i - VB], smask, tsh);
+          tab_dispatch<R, B>(x, op.ku, reinterpret_cast<const T2*>(at(&SmemMap::vts)) + tb.s0, tb.ns, pattern_fast(global_of(local_row(), m0, m1, sh) | cur_base, smask, tsh), pr);
         }
-      } else {
-        phase_apply<R, NR, B>(x, sph[op.idx], scls, Cs, e0s[op.idx], lt);
       }
     }
-    // The sweep's rotation scale m (-i)^K, then the rows straight to HBM:
-    // register row 2j (and 2j + 1 in the same 16 bytes for complex64) sits at
-    // global row gt ^ XOR of the layout's global offsets of the set bits of 2j.
-    // (One store body per form of the scale, so no join follows it.)
-    const R m = m_sweep;
-    const int K = k_sweep;
-    uint32_t go[B];
+    // The sweep's scale (real unless a rotation made an odd number of quarter
+    // turns or a bond left its phase), then the rows straight to HBM: chunk j
+    // of the thread sits at global row gt ^ XOR of the layout's global offsets
+    // of the set bits of j.
+    const T2 out_scale = *reinterpret_cast<const T2*>(at(&SmemMap::scale));
+    if (out_scale.y != R(0)) {
+      if constexpr (V == 2) {
+        const float2 c = dup(out_scale.x), s = dup(out_scale.y), ns = dup(-out_scale.y);
 #pragma unroll
-    for (int i = 0; i < B; ++i) go[i] = cur->goff[i];
-    auto store_rows = [&](auto scale) {
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        uint32_t g = gt;
-#pragma unroll
-        for (int i = 0; i < B - VB; ++i)
-          if ((j >> i) & 1) g ^= go[i + VB];
-        if constexpr (V == 2) {
-          const T2 v0 = scale(x[2 * j]), v1 = scale(x[2 * j + 1]);
-          *reinterpret_cast<float4*>(dst + HS_BCHK(g, a.N - 1, BS_REG_STATE)) = make_float4(v0.x, v0.y, v1.x, v1.y);
-        } else {
-          dst[HS_BCHK(g, a.N, BS_REG_STATE)] = scale(x[j]);
+        for (int j = 0; j < NJ; ++j) {
+          const float2 r = x.re[j], m = x.im[j];
+          x.re[j] = fma2(r, c, __fmul2_rn(m, ns));
+          x.im[j] = fma2(r, s, __fmul2_rn(m, c));
         }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) x.x[k] = cmul<T2, R>(x.x[k], out_scale.x, out_scale.y);
       }
-    };
+    } else if (out_scale.x != R(1)) {
+      if constexpr (V == 2) {
+        const float2 c = dup(out_scale.x);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          x.re[j] = __fmul2_rn(x.re[j], c);
+          x.im[j] = __fmul2_rn(x.im[j], c);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) x.x[k] = T2{x.x[k].x * out_scale.x, x.x[k].y * out_scale.x};
+      }
+    }
+    T2* dst = reinterpret_cast<T2*>(a.dst) + HS_BCHK(cur_state, a.n_rhs, BS_REG_STATE) * a.N;
+    const uint4 go4 = *reinterpret_cast<const uint4*>(lays[cur].L.goff);
+    const uint32_t go[4] = {go4.x, go4.y, go4.z, go4.w};
+    const uint32_t gt = global_of(local_row(), m0, m1, sh) | cur_base;
     // When the two lowest register bits are local bits 0 and 1 (complex64;
     // for complex128 register bit 0 is local bit 0) and the tile keeps those
     // bits contiguous, a thread's registers 4q .. 4q + 3 (2q, 2q + 1) are 32
     // consecutive bytes: one 32-byte store fills a whole sector.
     constexpr int WB = V == 2 ? 2 : 1;  // register bits inside a 32-byte store
-    auto store_wide = [&](auto scale) {
+    const uint32_t wide_bits = (1u << WB) - 1u;  // local bits that must be the lowest register bits
+    const bool wide = (lays[cur].L.reg & wide_bits) == wide_bits && (m0 & wide_bits) == wide_bits &&
+                      (reinterpret_cast<uintptr_t>(a.dst) & 31u) == 0;  // (states may be only 16-byte aligned)
+    if (wide) {
 #pragma unroll
-      for (int q = 0; q < (NR >> WB); ++q) {
+      for (int w = 0; w < (NR >> WB); ++w) {
         uint32_t g = gt;
 #pragma unroll
         for (int i = WB; i < B; ++i)
-          if (((q << WB) >> i) & 1) g ^= go[i];
+          if (((w << WB) >> i) & 1) g ^= go[i - VB];
         T2* p = dst + HS_BCHK(g, a.N - (1 << WB) + 1, BS_REG_STATE);
         if constexpr (V == 2) {
-          const T2 v0 = scale(x[4 * q]), v1 = scale(x[4 * q + 1]), v2 = scale(x[4 * q + 2]), v3 = scale(x[4 * q + 3]);
-          asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(v0.x), "f"(v0.y),
-                       "f"(v1.x), "f"(v1.y), "f"(v2.x), "f"(v2.y), "f"(v3.x), "f"(v3.y)
+          const float2 r0 = x.re[2 * w], i0 = x.im[2 * w], r1 = x.re[2 * w + 1], i1 = x.im[2 * w + 1];
+          asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(r0.x), "f"(i0.x),
+                       "f"(r0.y), "f"(i0.y), "f"(r1.x), "f"(i1.x), "f"(r1.y), "f"(i1.y)
                        : "memory");
         } else {
-          const T2 v0 = scale(x[2 * q]), v1 = scale(x[2 * q + 1]);
+          const T2 v0 = x.x[2 * w], v1 = x.x[2 * w + 1];
           asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "d"(v0.x), "d"(v0.y), "d"(v1.x), "d"(v1.y)
                        : "memory");
         }
       }
-    };
-    const uint32_t wide_bits = (1u << WB) - 1u;  // local bits that must be the lowest register bits
-    const bool wide = (cur->reg & wide_bits) == wide_bits && (m0 & wide_bits) == wide_bits &&
-                      (reinterpret_cast<uintptr_t>(a.dst) & 31u) == 0;  // (states may be only 16-byte aligned)
-    if (K == 0) {
-      auto sc = [&](T2 v) { return T2{v.x * m, v.y * m}; };
-      if (wide) store_wide(sc); else store_rows(sc);
     } else {
-      const R cr = K == 2 ? -m : R(0), ci = K == 1 ? -m : (K == 3 ? m : R(0));
-      auto sc = [&](T2 v) { return T2{fma(v.x, cr, -v.y * ci), fma(v.x, ci, v.y * cr)}; };
-      if (wide) store_wide(sc); else store_rows(sc);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        uint32_t g = gt;
+#pragma unroll
+        for (int i = 0; i < NJB; ++i)
+          if ((j >> i) & 1) g ^= go[i];
+        if constexpr (V == 2)
+          *reinterpret_cast<float4*>(dst + HS_BCHK(g, a.N - 1, BS_REG_STATE)) =
+              make_float4(x.re[j].x, x.im[j].x, x.re[j].y, x.im[j].y);
+        else
+          dst[HS_BCHK(g, a.N, BS_REG_STATE)] = x.x[j];
+      }
     }
+    if (!more) break;
   }
 }
 
 // FULL: the kernel with the TAB and general-rotation paths; sweeps without
-// them run the lighter instantiation (fewer live registers, no spills).  NT:
-// threads per CTA the instantiation is built for (2^(tile_bits - B); 512 for
-// 2^14-row complex64 tiles with five register bits, one CTA per SM).
+// them run the lighter instantiation.  NT: threads per CTA the instantiation
+// is built for (2^(tile_bits - B); 512 for 2^14-row complex64 tiles with five
+// register bits, one CTA per SM).
 template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512)>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const uint32_t u0 = blockIdx.x * uint32_t(a.units_per_cta);
-  const uint32_t u1 = min(uint32_t(a.n_units), u0 + uint32_t(a.units_per_cta));
-  qsweep_core<R, B, FULL>(a, u0, u1, smem_raw, true);
+  qsweep_core<R, B, FULL>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw, true);
 }
 
 template <typename R, int B, bool FULL>
@@ -824,8 +1107,8 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
     if (pref[mid] <= int(blockIdx.x)) lo = mid; else hi = mid - 1;
   }
   const Args& a = p.descs[p.lvl_desc[p.off + lo]];
-  const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_units, BS_BATCH_JOB));
-  qsweep_core<R, B, FULL>(a, u, u + 1, smem_raw, true);
+  const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_chunks, BS_BATCH_JOB));
+  qsweep_core<R, B, FULL>(a, u, u + 1, 1u, smem_raw, true);
 }
 
 using LFn = void (*)(LevelArgs);
@@ -885,16 +1168,27 @@ cudaError_t prepare_qsweep() {
 }
 
 size_t qsweep_smem_bytes(const Args& a, hs_dtype dt, int B) {
-  const size_t e = elem_bytes(dt), r = e / 2;
-  const size_t warps = size_t(1) << (a.tile_bits - B - 5);
-  const size_t head =
-      ((size_t(1) << a.tile_bits) + a.n_rot + a.n_vt + warps * a.n_phase) * e + warps * size_t(a.n_cls) * r;
-  return (head + 15) / 16 * 16 + sizeof(Op) * a.n_ops + sizeof(Layout) * a.n_lay + sizeof(Phase) * a.n_phase +
-         sizeof(PClass) * a.n_cls + sizeof(PTerm) * a.n_pterm + 16 + r * a.n_pterm + 16 + 12 * warps + a.n_ops + 16 +
-         192 * size_t(a.n_lay);
+  return smem_map(a, uint32_t(elem_bytes(dt)), 1u << (a.tile_bits - B)).total;
 }
 
-void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs) {
+// The most states of a tile a CTA runs back to back (a PHASE run's factors are
+// computed for the first only) that does not lengthen the longest CTA by more
+// than a fiftieth.
+int pick_rhs_chunk(int64_t tiles, int n_rhs, int slots) {
+  int best = 1;
+  int64_t best_len = 0;
+  for (int k = 1; k <= std::min(n_rhs, kMaxRhsChunk); k *= 2) {
+    const int64_t chunks = tiles * ((n_rhs + k - 1) / k);
+    const int64_t len = (chunks + slots - 1) / slots * k;
+    if (best_len == 0 || len * 50 <= best_len * 51) {
+      best = k;
+      best_len = best_len == 0 ? len : std::min(len, best_len);
+    }
+  }
+  return best;
+}
+
+void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs, int rhs_chunk) {
   const Plan& p = f->plan;
   a.src = psi;
   a.dst = psi;
@@ -907,7 +1201,9 @@ void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs) {
   a.n_terms_g = int(p.x.size()) * p.n_kinds;
   a.n_rhs = n_rhs;
   a.n_tiles_log2 = p.n_qubits - a.tile_bits;
-  a.n_units = (1 << a.n_tiles_log2) * n_rhs;
+  a.rhs_chunk = rhs_chunk;
+  a.rhs_chunks = (n_rhs + rhs_chunk - 1) / rhs_chunk;
+  a.n_chunks = (1 << a.n_tiles_log2) * a.rhs_chunks;
 }
 
 cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
@@ -935,23 +1231,23 @@ cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* d
   const Plan& p = f->plan;
   QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits);
   if (!fn || a.tile_bits - B < 5 || a.tile_bits > p.n_qubits) return cudaErrorInvalidValue;
-  fill_job(f, a, const_cast<void*>(src), n_rhs);
+  const size_t smem = qsweep_smem_bytes(a, f->dtype, B);
+  if (smem > kSweepSmemMax) return cudaErrorInvalidValue;
+  // One resident CTA per slot of the chip runs its share of the chunks back to
+  // back (its tables are loaded once).
+  const int threads = 1 << (a.tile_bits - B);
+  const int per_sm = std::max(1, std::min({32, 65536 / (128 * threads), int((kSmemPerSm) / (smem + 1024))}));
+  const int slots = kSMs * per_sm;
+  fill_job(f, a, const_cast<void*>(src), n_rhs, pick_rhs_chunk(int64_t(1) << (p.n_qubits - a.tile_bits), n_rhs, slots));
   a.dst = dst;
   if (rq) {
     a.rq = rq;
     a.cs = cs;
     a.n_terms_g = n_terms;
   }
-  // Several tiles per CTA once the grid is large (the per-CTA tables are then
-  // loaded once for them), up to eight, keeping at least four waves of two
-  // CTAs per SM (eight units per CTA measured 2.7% faster than four on the
-  // 24-qubit, 16-state MaxCut sweeps).
-  if (a.units_per_cta < 1) a.units_per_cta = std::max(1, std::min(8, a.n_units / (152 * 2 * 4)));
-  const size_t smem = qsweep_smem_bytes(a, f->dtype, B);
-  if (smem > kSweepSmemMax) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned((a.n_units + a.units_per_cta - 1) / a.units_per_cta), 1u, 1u);
-  cfg.blockDim = dim3(unsigned(1u << (a.tile_bits - B)), 1u, 1u);
+  cfg.gridDim = dim3(unsigned(std::min(a.n_chunks, slots)), 1u, 1u);
+  cfg.blockDim = dim3(unsigned(threads), 1u, 1u);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

@@ -23,6 +23,12 @@
 //          k a swap of partner rows;
 //   ROTN   a run of consecutive X-type single-qubit rotations on distinct
 //          register bits (they commute), applied back to back in that form;
+//   BOND   the terms XX, YY and ZZ of one qubit pair with one angle theta (they
+//          commute): exp(-i theta (XX + YY + ZZ)) = e^{-i theta} (I + w S), where
+//          S takes (x01, x10) to (x10 - x01, x01 - x10) and every other row to 0,
+//          w = (1 - e^{4 i theta}) / 2; the phase goes into the sweep's scale.
+//          10 real operations per pair of rows that change, none for the others,
+//          against 32 through a value table;
 //   DROT   a single diagonal term between non-diagonal ones: its rotation
 //          exp(-i theta (-1)^popcount(z & r)) from the build's FP64 (cos, sin);
 //   PHASE  a run of consecutive diagonal terms (x = 0) of such a factor: the
@@ -51,15 +57,17 @@ constexpr int kMaxPTerms = 320;
 constexpr int kMaxClasses = 256;
 constexpr int kMaxVt = 2048;   // value-table entries held in shared memory
 constexpr int kMaxB = 5;       // register bits per thread
+constexpr int kMaxBond = 64;
+constexpr int kMaxRhsChunk = 4;  // states of one tile a CTA runs back to back
 
-enum : uint8_t { OP_ROT = 0, OP_TAB = 1, OP_PHASE = 2, OP_LAYOUT = 3, OP_ROTN = 4, OP_DROT = 5 };
+enum : uint8_t { OP_ROT = 0, OP_TAB = 1, OP_PHASE = 2, OP_LAYOUT = 3, OP_ROTN = 4, OP_DROT = 5, OP_BOND = 6 };
 
 struct Op {
   uint8_t type;
-  uint8_t ku;     // ROT, TAB: the flip in register coordinates (TAB: 0 for a one-slot factor)
+  uint8_t ku;     // ROT, TAB, BOND: the flip in register coordinates (TAB: 0 for a one-slot factor)
   uint8_t zk;     // ROT: the register coordinates of z's bits in the tile
   uint8_t flags;  // ROT: bit 0 = fast path (y = 0 and z = 0); bits 1-2 = q with -i i^y = i^q
-  int16_t idx;    // ROT: rotation slot; TAB: table slot; PHASE: phase slot; LAYOUT: layout slot
+  int16_t idx;    // ROT: rotation slot; TAB: table slot; BOND: bond slot; PHASE: phase slot; LAYOUT: layout slot
   int16_t pad;
   uint32_t zthr;  // ROT: z's bits in the tile on thread positions (local-index mask)
   uint32_t zrest; // ROT: z's bits outside the tile (global mask)
@@ -68,21 +76,27 @@ struct Op {
   // byte i of (zthr, zrest) the rotation slot of register bit i.
 };
 
-struct Layout {
-  uint32_t reg;        // local-index mask of the register bits (register bit i = i-th lowest set bit)
-  uint32_t qoff[kMaxB];  // per register bit: XOR offset of the physical 16-byte chunk index
-  uint32_t goff[kMaxB];  // per register bit: global row offset (global image of the local bit)
-  int8_t thr[28];      // local positions of the thread-index bits, thread bit 0 first
-  int32_t n_thr;
+constexpr int kMaxNJB = 4;  // register bits that select a thread's 16-byte chunks
+
+struct alignas(16) Layout {
+  // Per register bit above those inside a chunk (complex64: above bit 0): XOR
+  // offset of the physical 16-byte chunk index, and the global row offset
+  // (global image of the local bit).
+  uint32_t qoff[kMaxNJB];
+  uint32_t goff[kMaxNJB];
   // A warp's rows (fixed warp bits, all register and lane bits) copied in
   // address order: chunk e = lane + 32 m of the warp's set lies at chunk
   // pdep(lane, wlo) ^ pdep(32 m, W) ^ (the warp's fixed chunk bits), W the
   // warp's chunk bits; mswz / mglob hold the swizzled chunk and global row
-  // of pdep(32 m, W).
+  // of pdep(32 m, W) for m = 1, 2, 4, 8 (both maps are linear over XOR).
+  uint32_t mswz[kMaxNJB];
+  uint32_t mglob[kMaxNJB];
+  uint32_t reg;        // local-index mask of the register bits (register bit i = i-th lowest set bit)
+  uint32_t g0;         // complex64: global row offset of register bit 0
+  int8_t thr[28];      // local positions of the thread-index bits, thread bit 0 first
+  int32_t n_thr;
   int8_t wlo[5];       // the five lowest chunk bits of W
   int8_t pad[3];
-  uint32_t mswz[1 << (kMaxB - 1)];
-  uint32_t mglob[1 << (kMaxB - 1)];
 };
 
 struct Rot {
@@ -105,6 +119,9 @@ struct Phase {
   uint32_t mu_mask;    // register patterns mu that have at least one class besides cls0
   int16_t mu_beg[(1 << kMaxB) + 1];  // per mu: first class (relative to cls0; mu = 0 starts
                                      // after the constant class), sentinel last
+  int16_t fac0;        // first of the run's factor slots (mu = 0, one per register bit, one per
+                       // further pattern present)
+  int16_t pad;
 };
 
 struct PClass {
@@ -132,17 +149,24 @@ struct Args {
   int n_rhs;
   int tile_bits;
   int n_tiles_log2;
-  int n_units;
-  int units_per_cta;
+  // Work is cut into chunks of up to rhs_chunk consecutive states of one tile
+  // (chunk q: tile q / rhs_chunks, states from (q % rhs_chunks) * rhs_chunk).
+  int rhs_chunk, rhs_chunks, n_chunks;
   uint32_t m0, m1;  // local index of global row r: (r & m0) | ((r >> sh) & m1)
   int sh;
   Runs rest;
-  int n_ops, n_lay, n_rot, n_tab, n_phase, n_cls, n_pterm, n_vt;
+  int n_ops, n_lay, n_rot, n_tab, n_phase, n_cls, n_pterm, n_vt, n_bond;
+  int n_fac;         // phase factor slots a thread has in shared memory
+  int fac_keep;      // 1: every PHASE run has slots of its own (kept for all states of a chunk);
+                     // 0: the runs share slots and their factors are computed on each use
+  int last_lay;      // index of the last LAYOUT op
+  int free_local;    // 1: the last layout's warp bits are the first one's
   int full;          // 1 if a TAB op or a rotation other than tan form occurs (the larger kernel)
   Op ops[kMaxOps];
   Layout lay[kMaxLayouts];
   Rot rot[kMaxRot];
   Tab tab[kMaxTab];
+  int32_t bond[kMaxBond];  // index of the bond's angle records
   Phase ph[kMaxPhase];
   PClass cls[kMaxClasses];
   PTerm pt[kMaxPTerms];
@@ -153,6 +177,40 @@ struct Args {
 // chunks a quarter-warp touches over distinct 16-byte bank groups.
 __host__ __device__ __forceinline__ uint32_t swz(uint32_t c) {
   return c ^ (((c >> 3) ^ (c >> 6) ^ (c >> 9) ^ (c >> 12) ^ (c >> 15)) & 7u);
+}
+
+// The register patterns mu of two or more bits among those present, by where
+// they lie: inside the lower group of register bits (0 .. (B + 1) / 2 - 1),
+// inside the upper group (in coordinates of that group for lower / upper), or
+// across the groups.  A set of patterns is a mask with bit mu.
+template <int B>
+__host__ __device__ __forceinline__ uint32_t lower_patterns(uint32_t mu_mask) {
+  uint32_t m = 0;
+  for (int mu = 3; mu < (1 << ((B + 1) / 2)); ++mu)
+    if (mu & (mu - 1)) m |= 1u << mu;
+  return mu_mask & m;
+}
+template <int B>
+__host__ __device__ __forceinline__ uint32_t upper_patterns(uint32_t mu_mask) {
+  constexpr int B1 = (B + 1) / 2;
+  uint32_t m = 0;
+  for (int nu = 3; nu < (1 << (B - B1)); ++nu)
+    if ((nu & (nu - 1)) && ((mu_mask >> (nu << B1)) & 1u)) m |= 1u << nu;
+  return m;
+}
+template <int B>
+__host__ __device__ __forceinline__ uint32_t inside_patterns(uint32_t mu_mask) {
+  constexpr int B1 = (B + 1) / 2;
+  uint32_t m = 0;
+  for (int nu = 3; nu < (1 << (B - B1)); ++nu)
+    if (nu & (nu - 1)) m |= 1u << (nu << B1);
+  return lower_patterns<B>(mu_mask) | (mu_mask & m);
+}
+template <int B>
+__host__ __device__ __forceinline__ uint32_t across_patterns(uint32_t mu_mask) {
+  uint32_t m = ~1u;
+  for (int i = 0; i < B; ++i) m &= ~(1u << (1 << i));
+  return mu_mask & m & ~inside_patterns<B>(0xffffffffu);
 }
 
 // Host planner: the ops of a fused sweep (factors in order, two-run local mask)
@@ -175,11 +233,15 @@ bool plan_qsweep_runs(const hs_factors* f, const std::vector<int>& factors, uint
 size_t qsweep_smem_bytes(const Args& a, hs_dtype dt, int B);
 
 // The job-dependent fields of a descriptor: state (evolved in place), the
-// factor set's angle records and value tables, and the unit count (tiles of
-// the planned local mask times n_rhs states).
-void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs);
+// factor set's angle records and value tables, and the chunks of work (tiles
+// of the planned local mask times n_rhs states, rhs_chunk states at a time).
+void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs, int rhs_chunk);
 
-// One level of a batch of register sweeps: CTA c runs unit c - prefix[e] of
+// States per chunk for a launch of `tiles` tiles of n_rhs states on `slots`
+// resident CTAs.
+int pick_rhs_chunk(int64_t tiles, int n_rhs, int slots);
+
+// One level of a batch of register sweeps: CTA c runs chunk c - prefix[e] of
 // descriptor lvl_desc[off + e], e the last entry with prefix[off + e] <= c.
 struct LevelArgs {
   const Args* descs;
