@@ -215,8 +215,10 @@ struct hs_batch {
     int* d_lvl_desc = nullptr;
     int* d_lvl_prefix = nullptr;
   };
-  std::vector<hs::q::Args> qdescs;
-  hs::q::Args* d_qdescs = nullptr;
+  std::vector<hs::q::Args> qdescs;  // until the tables are uploaded
+  hs::q::Hdr* d_qdescs = nullptr;
+  unsigned char* d_images = nullptr;  // records, templates and images of every descriptor
+  int n_images = 0;
   std::vector<QGroup> qgroups;
 };
 
@@ -225,7 +227,8 @@ namespace {
 void batch_release(hs_batch* b, cudaStream_t s) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
-  void* bufs[] = {b->d_jobs, b->d_sweeps, b->d_facs, b->d_lvl_sweep, b->d_lvl_prefix, b->d_qdescs};
+  void* bufs[] = {b->d_jobs, b->d_sweeps, b->d_facs, b->d_lvl_sweep, b->d_lvl_prefix, b->d_qdescs,
+                  b->d_images};
   for (void* p : bufs)
     if (p) cudaFreeAsync(p, s);
   for (auto& g : b->qgroups) {
@@ -247,7 +250,17 @@ int upload_tables(hs_batch* b, cudaStream_t s) {
   if (b->uploaded) return HS_OK;
   cudaError_t e;
   if (b->reg) {
-    e = upload(&b->d_qdescs, b->qdescs, s);
+    hs::q::Images im(b->dtype, b->reg_bits);
+    for (const hs::q::Args& a : b->qdescs) im.add(a);
+    b->n_images = im.count();
+    e = hs::pool_malloc(reinterpret_cast<void**>(&b->d_images), std::max<size_t>(1, im.device_bytes()), s);
+    if (e == cudaSuccess && b->n_images) {
+      const std::vector<unsigned char> blob = im.blob(b->d_images);
+      e = cudaMemcpyAsync(b->d_images, blob.data(), blob.size(), cudaMemcpyHostToDevice, s);
+      std::vector<hs::q::Hdr> hd;
+      for (size_t i = 0; i < b->qdescs.size(); ++i) hd.push_back(im.header(b->qdescs[i], int(i), b->d_images));
+      if (e == cudaSuccess) e = upload(&b->d_qdescs, hd, s);
+    }
     for (auto& g : b->qgroups)
       if (e == cudaSuccess && (e = upload(&g.d_lvl_desc, g.lvl_desc, s)) == cudaSuccess)
         e = upload(&g.d_lvl_prefix, g.lvl_prefix, s);
@@ -273,10 +286,15 @@ int enqueue_batch(hs_batch* b, cudaStream_t s) {
     if (rc != HS_OK) return rc;
   }
   if (b->reg) {
+    const cudaError_t e0 = hs::q::launch_fill(b->dtype, b->d_images, b->n_images, s);
+    if (e0 != cudaSuccess)
+      return hs::report_error(HS_ECUDA, std::string("batch table launch: ") + cudaGetErrorString(e0));
+    bool early = false;  // (the tables are complete before the first level starts)
     for (const hs_batch::QGroup& g : b->qgroups)
       for (const hs_batch::Level& L : g.levels) {
         hs::q::LevelArgs a{b->d_qdescs, g.d_lvl_desc, g.d_lvl_prefix, L.off, L.count, uint32_t(g.prefix_smem)};
-        cudaError_t e = hs::q::launch_qlevel(b->dtype, b->reg_bits, L.full, g.tile_bits, a, L.ctas, g.smem, s);
+        cudaError_t e = hs::q::launch_qlevel(b->dtype, b->reg_bits, L.full, g.tile_bits, a, L.ctas, g.smem, early, s);
+        early = true;
         if (e != cudaSuccess)
           return hs::report_error(HS_ECUDA, std::string("batch level launch: ") + cudaGetErrorString(e));
       }
@@ -441,7 +459,7 @@ int create_reg_batch(const hs_batch_job* jobs, size_t n_jobs, const hs_batch_opt
       g.levels.push_back(L);
     }
     g.prefix_smem = (smem + 15) / 16 * 16;
-    g.smem = g.prefix_smem + size_t(max_count) * sizeof(int);
+    g.smem = g.prefix_smem + hs::q::kHdrSmem + size_t(max_count) * sizeof(int);
     if (g.smem > hs::kSweepSmemMax) return hs::report_error(HS_EINVAL, "batch needs more shared memory than a CTA has");
     b->levels.insert(b->levels.end(), g.levels.begin(), g.levels.end());  // for hs_batch_info
     b->qgroups.push_back(std::move(g));

@@ -24,8 +24,8 @@
 // every op works on pairs with the two-element FP32 instructions (half the
 // instructions of the scalar form for the same operations), and the phase
 // factors are produced by one loop with one sincospi.  On the 24-qubit MaxCut
-// instance with 16 states a sweep went from 2.09 to 1.51 ms; a periodic
-// 22-qubit Heisenberg chain with 2 states (BOND ops) from 3.85 to 1.72 ms for
+// instance with 16 states a sweep went from 2.09 to 1.46 ms; a periodic
+// 22-qubit Heisenberg chain with 2 states (BOND ops) from 3.85 to 1.67 ms for
 // 20 steps.  Registers matter as much: the tiles leave little L1, so a spilled
 // register costs an L2 round trip (52 local loads per warp and tile made the
 // 1.51 ms sweep a 6.2 ms one).
@@ -44,6 +44,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "counters.h"
 #include "hs_internal.h"
@@ -199,19 +200,30 @@ __device__ __forceinline__ void rot_ku(Rows<R, B>& x, R c, R s, bool fast, int q
     if (flip) flip_pairs<R, KU>(x);
     return;
   }
-  const R qx = (q == 0) ? s : (q == 2 ? -s : R(0));
-  const R qy = (q == 1) ? s : (q == 3 ? -s : R(0));
+  // (i^q s as one component, real or imaginary; a row's sign from z's bits by
+  // XOR with one mask per bit, so that no table of signs fills the registers)
+  const bool imag = q & 1;
+  uint32_t zm[B];
+#pragma unroll
+  for (int i = 0; i < B; ++i) zm[i] = (zk >> i) & 1u;
+  const R s0 = flip_sign(s, uint32_t(sb) ^ uint32_t(q >> 1));
+  auto coef = [&](int k) {  // of a row whose partner is row k
+    uint32_t p = 0;
+#pragma unroll
+    for (int i = 0; i < B; ++i)
+      if ((k >> i) & 1) p ^= zm[i];
+    return flip_sign(s0, p);
+  };
 #pragma unroll
   for (int k = 0; k < (1 << B); ++k) {
     if (k & HB) continue;
     const int k2 = k ^ KU;
     const T2 b1 = x.get(k), b2 = x.get(k2);
-    // row k pairs with column k2 (sign of r_k2), row k2 with column k (sign of r_k)
-    const R sk = (sb ^ parity(zk & uint32_t(k2))) ? R(-1) : R(1);
-    const R sk2 = (sb ^ parity(zk & uint32_t(k))) ? R(-1) : R(1);
-    const R ax = sk * qx, ay = sk * qy, bx = sk2 * qx, by = sk2 * qy;
-    x.set(k, T2{fma(ax, b2.x, fma(-ay, b2.y, c * b1.x)), fma(ax, b2.y, fma(ay, b2.x, c * b1.y))});
-    x.set(k2, T2{fma(bx, b1.x, fma(-by, b1.y, c * b2.x)), fma(bx, b1.y, fma(by, b1.x, c * b2.y))});
+    const R c1 = coef(k2), c2 = coef(k);
+    // (x, y) i = (-y, x)
+    const R u1 = imag ? -b2.y : b2.x, v1 = imag ? b2.x : b2.y, u2 = imag ? -b1.y : b1.x, v2 = imag ? b1.x : b1.y;
+    x.set(k, T2{fma(c1, u1, c * b1.x), fma(c1, v1, c * b1.y)});
+    x.set(k2, T2{fma(c2, u2, c * b2.x), fma(c2, v2, c * b2.y)});
   }
 }
 
@@ -304,19 +316,12 @@ __device__ __forceinline__ void tab_ku(Rows<R, B>& x, const typename C2<R>::T* t
       r2.y = fma(c0.x, b2.y, fma(c0.y, b2.x, fma(c1.x, b1.y, c1.y * b1.x)));
       x.set(k, r1);
       x.set(k2, r2);
+      // (keeps the loads of later rows below: hoisted, they take more registers
+      // than there are)
+      asm volatile("" ::: "memory");
     }
   }
 }
-
-// An op's coefficients: ROTN the tan(theta') of register bits 0 .. 4, ROT and
-// DROT (cos, sin) or (tan, 0), BOND w; `swap` the register bits (ROTN) or the
-// flag (ROT) of odd quarter turns.
-template <typename R>
-struct alignas(16) Coef {
-  R v[5];
-  uint32_t swap;
-  uint32_t pad[sizeof(R) == 4 ? 2 : 1];
-};
 
 // ROTN: commuting X rotations on distinct single register bits (tan form, see
 // ROT), the slot of register bit i in byte i of (zthr, zrest).  The rows of
@@ -325,10 +330,6 @@ struct alignas(16) Coef {
 // flips) is therefore one straight-line body (24-qubit MaxCut: 87.5 ms with a
 // branch per bit).  The odd-k swaps follow the whole run (every factor of the
 // run is a function of its own X, so they commute).
-__device__ __forceinline__ int rotn_slot(const Op& op, int i) {
-  return int((i < 4 ? (op.zthr >> (8 * i)) : (op.zrest >> (8 * (i - 4)))) & 0xffu);
-}
-
 template <typename R, int B, int I, bool ALL>
 __device__ __forceinline__ void rotn_bits(Rows<R, B>& x, uint32_t ku, const R (&t)[5]) {
   if constexpr (I < B) {
@@ -468,20 +469,23 @@ __device__ __forceinline__ void phase_factor(const Phase& P, const ClassC<R>* cw
   sincospi_r(e, sn, cn);
 }
 
-// A[k], k over N register bits, from A[0] and the bits' (cos, sin): f_i(0) =
+// A[k], k over N register bits, from A[0] and the bits' (cos, sin) in the slots
+// at cs (read one at a time: few registers are left beside the rows): f_i(0) =
 // cos - i sin, f_i(1) = cos + i sin; then the patterns (in coordinates of the
 // N bits) listed in `pats`, from the slots at `f`.
 template <typename T2, typename R, int N>
 __device__ __forceinline__ void group_values(T2 (&A)[1 << N], const T2* cs, uint32_t pats, const T2*& f, int nt) {
 #pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int i = 0; i < N; ++i) {
+    const T2 c = cs[i * nt];
 #pragma unroll
     for (int k = 0; k < (1 << i); ++k) {
       const T2 p = A[k];
-      const R ac = p.x * cs[i].x, bs = p.y * cs[i].y, bc = p.y * cs[i].x, as = p.x * cs[i].y;
+      const R ac = p.x * c.x, bs = p.y * c.y, bc = p.y * c.x, as = p.x * c.y;
       A[k] = T2{ac + bs, bc - as};
       A[k + (1 << i)] = T2{ac - bs, bc + as};
     }
+  }
 #pragma unroll 1
   for (uint32_t r = pats; r; r &= r - 1u, f += nt) {
     const int mu = __ffs(r) - 1;
@@ -497,14 +501,11 @@ __host__ __device__ constexpr int lower_bits(int B) { return (B + 1) / 2; }
 template <int B>
 __device__ __forceinline__ void phase_apply(Rows<float, B>& x, uint32_t mu_mask, const float2* fac, int nt) {
   constexpr int B1 = lower_bits(B), B2 = B - B1;
-  float2 cs[B];
-#pragma unroll
-  for (int i = 0; i < B; ++i) cs[i] = fac[(1 + i) * nt];
   const float2* f = fac + (1 + B) * nt;
   {
     float2 A[1 << B1];
     A[0] = fac[0];
-    group_values<float2, float, B1>(A, cs, lower_patterns<B>(mu_mask), f, nt);
+    group_values<float2, float, B1>(A, fac + nt, lower_patterns<B>(mu_mask), f, nt);
 #pragma unroll
     for (int a = 0; a < (1 << (B1 - 1)); ++a) {
       const float2 c = make_float2(A[2 * a].x, A[2 * a + 1].x), s = make_float2(A[2 * a].y, A[2 * a + 1].y), ns = neg2(s);
@@ -520,7 +521,7 @@ __device__ __forceinline__ void phase_apply(Rows<float, B>& x, uint32_t mu_mask,
   {
     float2 A[1 << B2];
     A[0] = make_float2(1.0f, 0.0f);
-    group_values<float2, float, B2>(A, cs + B1, upper_patterns<B>(mu_mask), f, nt);
+    group_values<float2, float, B2>(A, fac + (1 + B1) * nt, upper_patterns<B>(mu_mask), f, nt);
 #pragma unroll
     for (int b = 0; b < (1 << B2); ++b) {
       const float2 c = dup(A[b].x), s = dup(A[b].y), ns = dup(-A[b].y);
@@ -554,15 +555,12 @@ __device__ __forceinline__ void pattern_apply(Rows<float, B>& x, int mu, float2 
 template <int B>
 __device__ __forceinline__ void phase_apply(Rows<double, B>& x, uint32_t mu_mask, const double2* fac, int nt) {
   constexpr int B1 = lower_bits(B), B2 = B - B1;
-  double2 cs[B];
-#pragma unroll
-  for (int i = 0; i < B; ++i) cs[i] = fac[(1 + i) * nt];
   const double2* f = fac + (1 + B) * nt;
   double2 A[1 << B1], C[1 << B2];
   A[0] = fac[0];
-  group_values<double2, double, B1>(A, cs, lower_patterns<B>(mu_mask), f, nt);
+  group_values<double2, double, B1>(A, fac + nt, lower_patterns<B>(mu_mask), f, nt);
   C[0] = make_double2(1.0, 0.0);
-  group_values<double2, double, B2>(C, cs + B1, upper_patterns<B>(mu_mask), f, nt);
+  group_values<double2, double, B2>(C, fac + (1 + B1) * nt, upper_patterns<B>(mu_mask), f, nt);
 #pragma unroll
   for (int k = 0; k < (1 << B); ++k) x.x[k] = cmul<double2, double>(x.x[k], A[k & ((1 << B1) - 1)].x, A[k & ((1 << B1) - 1)].y);
 #pragma unroll
@@ -613,47 +611,133 @@ __device__ __forceinline__ void phase_op(Rows<R, B>& x, const Phase& P, const Cl
   }
 }
 
-// Byte offsets of a CTA's tables in shared memory (the tile comes first).
-struct SmemMap {
-  uint32_t ops, lays, fac, vts, e0s, cw, ph, cls, pt, thpi, clane, scale, total;
+// ---------------------------------------------------------------------------
+// Coefficients.  rec: the term records of the op (ROTN: one per register bit).
+// m, kq and ph collect the sweep's scale: the product of the fast rotations'
+// cos(theta') and quarter turns (-i)^k and of the bonds' phases e^{-i theta}.
+// ---------------------------------------------------------------------------
+struct Records {
+  const double* rq;
+  const double* cs;
+  int n;
 };
 
-// An op with its coefficients; a layout with the local row (x) and the
-// swizzled chunk (y) that a lane index (0 .. 31) and a warp index (32 ..)
-// deposit: a thread's register row 0 is the XOR of the two.
 template <typename R>
-struct OpRec {
-  Op op;
-  Coef<R> c;
-};
-struct LayRec {
-  Layout L;
-  uint2 dep[48];
-};
-
-__host__ __device__ __forceinline__ SmemMap smem_map(const Args& a, uint32_t e, uint32_t nt) {
-  SmemMap m;
-  uint32_t o = e << a.tile_bits;
-  auto take = [&](uint32_t bytes) {
-    const uint32_t at = o;
-    o += (bytes + 15u) & ~15u;
-    return at;
+__device__ __forceinline__ Coef<R> coef_of(const Op& op, const int32_t* rec, const Records& t, double& m, double& ph,
+                                           int& kq) {
+  Coef<R> c{};
+  // A fast rotation (y = 0, z = 0): tan(theta') of the factor build's record.
+  auto take = [&](int e, R& v) {
+    const double* q = t.rq + 4 * HS_BCHK(e, t.n, BS_REG_TERM);
+    v = R(q[0]);
+    m *= q[2];
+    const int k = int(q[1]);
+    kq += k;
+    return uint32_t(k & 1);
   };
-  const uint32_t warps = nt >> 5;
-  m.ops = take((e == 8 ? sizeof(OpRec<float>) : sizeof(OpRec<double>)) * a.n_ops);
-  m.lays = take(sizeof(LayRec) * a.n_lay);
-  m.fac = take(e * nt * a.n_fac);
-  m.vts = take(e * a.n_vt);
-  m.e0s = take(e * warps * a.n_phase);
-  m.cw = take(e * warps * a.n_cls);  // sizeof(ClassC<R>) = the element size
-  m.ph = take(sizeof(Phase) * a.n_phase);
-  m.cls = take(sizeof(PClass) * a.n_cls);
-  m.pt = take(sizeof(PTerm) * a.n_pterm);
-  m.thpi = take((e / 2) * a.n_pterm);
-  m.clane = take(48 * 4);
-  m.scale = take(e);
-  m.total = o;
-  return m;
+  if (op.type == OP_ROTN) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      if ((op.ku >> i) & 1) c.swap |= take(rec[i], c.v[i]) << i;
+  } else if (op.type == OP_ROT && (op.flags & 1)) {
+    c.swap = take(rec[0], c.v[0]);
+  } else if (op.type == OP_ROT || op.type == OP_DROT) {
+    const double* p = t.cs + 2 * HS_BCHK(rec[0], t.n, BS_REG_TERM);
+    c.v[0] = R(p[0]);
+    c.v[1] = R(p[1]);
+  } else if (op.type == OP_BOND) {
+    // w = (1 - e^{4 i theta}) / 2 = sin(2 theta) (sin(2 theta) - i cos(2 theta))
+    const int64_t e = HS_BCHK(rec[0], t.n, BS_REG_TERM);
+    const double cs = t.cs[2 * e], sn = t.cs[2 * e + 1];
+    const double s2 = 2.0 * cs * sn, c2 = fma(-2.0 * sn, sn, 1.0);
+    c.v[0] = R(s2 * s2);
+    c.v[1] = R(-s2 * c2);
+    ph += t.rq[4 * e + 3];  // theta / pi
+  }
+  return c;
+}
+
+__device__ __forceinline__ void sum_scale(double& m, double& ph, int& kq) {
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    m *= __shfl_xor_sync(0xffffffffu, m, o);
+    ph += __shfl_xor_sync(0xffffffffu, ph, o);
+    kq += __shfl_xor_sync(0xffffffffu, kq, o);
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ typename C2<R>::T scale_of(double m, double ph, int kq) {
+  using T2 = typename C2<R>::T;
+  const double u0 = ph + 0.5 * double(kq & 3), u = u0 - 2.0 * rint(0.5 * u0);
+  double sn, cn;
+  sincospi(u, &sn, &cn);
+  return T2{R(m * cn), R(-m * sn)};
+}
+
+// The records of op oi of a descriptor.
+__host__ __device__ __forceinline__ void records_of(const Args& a, const Op& op, int32_t (&rec)[5]) {
+  for (int i = 0; i < 5; ++i) rec[i] = 0;
+  if (op.type == OP_ROTN) {
+    for (int i = 0; i < 5; ++i)
+      if ((op.ku >> i) & 1) rec[i] = a.rot[rotn_slot(op, i)].cs;
+  } else if (op.type == OP_ROT || op.type == OP_DROT) {
+    rec[0] = a.rot[op.idx].cs;
+  } else if (op.type == OP_BOND) {
+    rec[0] = a.bond[op.idx];
+  }
+}
+
+// A descriptor's tables, by the whole CTA (complete after the next barrier).
+template <typename R, int B>
+__device__ __forceinline__ void make_tables(const Args& a, const SmemMap& sm, unsigned char* smem_raw) {
+  using T2 = typename C2<R>::T;
+  constexpr int VB = sizeof(T2) == 8 ? 1 : 0;  // register bits inside a 16-byte chunk
+  const int NT = blockDim.x;
+  const uint32_t tid = threadIdx.x;
+  OpRec<R>* ops = reinterpret_cast<OpRec<R>*>(smem_raw + sm.ops);
+  LayRec* lays = reinterpret_cast<LayRec*>(smem_raw + sm.lays);
+  auto copy_words = [&](void* dst, const void* src, size_t bytes) {
+    const uint32_t* s4 = static_cast<const uint32_t*>(src);
+    uint32_t* d4 = static_cast<uint32_t*>(dst);
+    for (uint32_t w = tid; w < bytes / 4; w += NT) d4[w] = s4[w];
+  };
+  for (int i = 0; i < a.n_lay; ++i) copy_words(&lays[i].L, a.lay + i, sizeof(Layout));
+  copy_words(smem_raw + sm.tabs, a.tab, sizeof(Tab) * a.n_tab);
+  copy_words(smem_raw + sm.ph, a.ph, sizeof(Phase) * a.n_phase);
+  copy_words(smem_raw + sm.cls, a.cls, sizeof(PClass) * a.n_cls);
+  copy_words(smem_raw + sm.pt, a.pt, sizeof(PTerm) * a.n_pterm);
+  for (int e = tid; e < 48 * a.n_lay; e += NT) {
+    const int li = e / 48, j = e - 48 * li;
+    const uint32_t d = deposit_index(a.lay[li], j);
+    lays[li].dep[j] = make_uint2(d, swz(d >> VB));
+  }
+  uint32_t* clane = reinterpret_cast<uint32_t*>(smem_raw + sm.clane);
+  for (int j = tid; j < 48; j += NT) clane[j] = copy_index(a.lay[a.ops[0].idx], j, VB);
+  R* thpi = reinterpret_cast<R*>(smem_raw + sm.thpi);
+  for (int t = tid; t < a.n_pterm; t += NT) thpi[t] = R(a.rq[4 * HS_BCHK(a.pt[t].th, a.n_terms_g, BS_REG_TERM) + 3]);
+  T2* vts = reinterpret_cast<T2*>(smem_raw + sm.vts);
+  for (int t = 0; t < a.n_tab; ++t) {
+    const T2* g = reinterpret_cast<const T2*>(a.vt) + a.tab[t].vt0;
+    const int s0 = a.tab[t].s0, n = a.tab[t].n;
+    for (int e = tid; e < n; e += NT) vts[s0 + e] = g[HS_BCHK(a.tab[t].vt0 + e, a.n_vt_g, BS_REG_VT) - a.tab[t].vt0];
+  }
+  // One warp makes the coefficients and the scale, in FP64: the FP64 pipe takes
+  // tens of cycles per warp instruction, so the others stay off it.
+  if (tid < 32) {
+    double m = 1.0, ph = 0.0;
+    int kq = 0;
+    const Records t{a.rq, a.cs, a.n_terms_g};
+    for (int oi = tid; oi < a.n_ops; oi += 32) {
+      const Op op = a.ops[oi];
+      int32_t rec[5];
+      records_of(a, op, rec);
+      ops[oi].op = op;
+      ops[oi].c = coef_of<R>(op, rec, t, m, ph, kq);
+    }
+    sum_scale(m, ph, kq);
+    if (tid == 0) *reinterpret_cast<T2*>(smem_raw + sm.scale) = scale_of<R>(m, ph, kq);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -668,10 +752,12 @@ __host__ __device__ __forceinline__ SmemMap smem_map(const Args& a, uint32_t e, 
 // starts copying its rows of the CTA's next state or tile, which land while
 // the current one finishes in registers and goes straight back to HBM.
 // ---------------------------------------------------------------------------
-template <typename R, int B, bool FULL>
-__device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t q1, uint32_t stride,
-                                            unsigned char* smem_raw, bool pdl) {
+// D: Args (the tables are made here) or Hdr (they are copied from the image).
+template <typename R, int B, bool FULL, typename D>
+__device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1, uint32_t stride,
+                                            unsigned char* smem_raw) {
   using T2 = typename C2<R>::T;
+  constexpr bool kImage = std::is_same_v<D, Hdr>;
   constexpr int NR = 1 << B;
   constexpr int V = 16 / int(sizeof(T2));  // rows per 16-byte chunk (2 for complex64)
   constexpr int VB = V == 2 ? 1 : 0;       // register bits inside a chunk
@@ -682,114 +768,28 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
   const int sh = a.sh;
   const int warp = tid >> 5, lane = tid & 31;
 
-  const SmemMap sm = smem_map(a, sizeof(T2), NT);
+  SmemMap sm;
+  int first_lay;
+  if constexpr (kImage) {
+    sm = a.sm;
+    first_lay = a.first_lay;
+  } else {
+    sm = smem_map(a, sizeof(T2), NT);
+    first_lay = a.ops[0].idx;  // the first op is always a layout
+  }
   auto at = [&](uint32_t SmemMap::* field) -> unsigned char* { return smem_raw + sm.*field; };
   T2* tile = reinterpret_cast<T2*>(smem_raw);
-  OpRec<R>* ops = reinterpret_cast<OpRec<R>*>(smem_raw + sm.ops);
-  LayRec* lays = reinterpret_cast<LayRec*>(smem_raw + sm.lays);
-  T2* fac = reinterpret_cast<T2*>(smem_raw + sm.fac) + tid;
+  OpRec<R>* ops = reinterpret_cast<OpRec<R>*>(at(&SmemMap::ops));
+  LayRec* lays = reinterpret_cast<LayRec*>(at(&SmemMap::lays));
+  T2* fac = reinterpret_cast<T2*>(at(&SmemMap::fac)) + tid;
 
   // Per-CTA tables (written by launches that completed before this grid began).
-  {
-    auto copy_words = [&](void* dst, const void* src, size_t bytes) {
-      const uint32_t* s4 = static_cast<const uint32_t*>(src);
-      uint32_t* d4 = static_cast<uint32_t*>(dst);
-      for (uint32_t w = tid; w < bytes / 4; w += NT) d4[w] = s4[w];
-    };
-    for (int i = 0; i < a.n_lay; ++i) copy_words(&lays[i].L, a.lay + i, sizeof(Layout));
-    copy_words(smem_raw + sm.ph, a.ph, sizeof(Phase) * a.n_phase);
-    copy_words(smem_raw + sm.cls, a.cls, sizeof(PClass) * a.n_cls);
-    copy_words(smem_raw + sm.pt, a.pt, sizeof(PTerm) * a.n_pterm);
-  }
-  for (int e = tid; e < 48 * a.n_lay; e += NT) {
-    const int li = e / 48, j = e - 48 * li;
-    const Layout& L = a.lay[li];
-    uint32_t d = 0;
-    if (j < 32)
-      for (int i = 0; i < 5 && i < L.n_thr; ++i) d |= uint32_t((j >> i) & 1) << L.thr[i];
-    else
-      for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
-    lays[li].dep[j] = make_uint2(d, swz(d >> VB));
-  }
-  // The local rows that a lane and a warp index deposit in the copies of the
-  // first layout's rows in address order.
-  uint32_t* clane_s = reinterpret_cast<uint32_t*>(smem_raw + sm.clane);
-  for (int j = tid; j < 48; j += NT) {
-    const Layout& L = a.lay[a.ops[0].idx];
-    uint32_t d = 0;
-    if (j < 32) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) d |= uint32_t((j >> k) & 1) << (L.wlo[k] + VB);
-    } else {
-      for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
-    }
-    clane_s[j] = d;
-  }
-  R* thpi_s = reinterpret_cast<R*>(smem_raw + sm.thpi);
-  for (int t = tid; t < a.n_pterm; t += NT) thpi_s[t] = R(a.rq[4 * HS_BCHK(a.pt[t].th, a.n_terms_g, BS_REG_TERM) + 3]);
-  T2* vts = reinterpret_cast<T2*>(smem_raw + sm.vts);
-  for (int t = 0; t < a.n_tab; ++t) {
-    const T2* g = reinterpret_cast<const T2*>(a.vt) + a.tab[t].vt0;
-    const int s0 = a.tab[t].s0, n = a.tab[t].n;
-    for (int e = tid; e < n; e += NT) vts[s0 + e] = g[HS_BCHK(a.tab[t].vt0 + e, a.n_vt_g, BS_REG_VT) - a.tab[t].vt0];
-  }
-  // Coefficients of every op, and the sweep's scale (the same for every tile):
-  // the product of the fast rotations' cos(theta') and quarter turns (-i)^k
-  // and of the bonds' phases e^{-i theta}.  One warp does this, in FP64: the
-  // FP64 pipe takes tens of cycles per warp instruction, so the others stay
-  // off it.
-  if (warp == 0) {
-    double m = 1.0, ph = 0.0;
-    int kq = 0;
-    // A fast rotation (y = 0, z = 0): tan(theta') of the factor build's record.
-    auto take = [&](int rot, R& t) {
-      const double* q = a.rq + 4 * HS_BCHK(a.rot[rot].cs, a.n_terms_g, BS_REG_TERM);
-      t = R(q[0]);
-      m *= q[2];
-      const int k = int(q[1]);
-      kq += k;
-      return uint32_t(k & 1);
-    };
-    for (int oi = lane; oi < a.n_ops; oi += 32) {
-      const Op& op = a.ops[oi];
-      Coef<R> c;
-      c.swap = 0;
-#pragma unroll
-      for (int i = 0; i < 5; ++i) c.v[i] = R(0);
-      if (op.type == OP_ROTN) {
-#pragma unroll
-        for (int i = 0; i < B; ++i)
-          if ((op.ku >> i) & 1) c.swap |= take(rotn_slot(op, i), c.v[i]) << i;
-      } else if (op.type == OP_ROT && (op.flags & 1)) {
-        c.swap = take(op.idx, c.v[0]);
-      } else if (op.type == OP_ROT || op.type == OP_DROT) {
-        const double* p = a.cs + 2 * HS_BCHK(a.rot[op.idx].cs, a.n_terms_g, BS_REG_TERM);
-        c.v[0] = R(p[0]);
-        c.v[1] = R(p[1]);
-      } else if (op.type == OP_BOND) {
-        // w = (1 - e^{4 i theta}) / 2 = sin(2 theta) (sin(2 theta) - i cos(2 theta))
-        const int64_t e = HS_BCHK(a.bond[op.idx], a.n_terms_g, BS_REG_TERM);
-        const double cs = a.cs[2 * e], sn = a.cs[2 * e + 1];
-        const double s2 = 2.0 * cs * sn, c2 = fma(-2.0 * sn, sn, 1.0);
-        c.v[0] = R(s2 * s2);
-        c.v[1] = R(-s2 * c2);
-        ph += a.rq[4 * e + 3];  // theta / pi
-      }
-      ops[oi].op = op;
-      ops[oi].c = c;
-    }
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) {
-      m *= __shfl_xor_sync(0xffffffffu, m, o);
-      ph += __shfl_xor_sync(0xffffffffu, ph, o);
-      kq += __shfl_xor_sync(0xffffffffu, kq, o);
-    }
-    if (lane == 0) {
-      const double u0 = ph + 0.5 * double(kq & 3), u = u0 - 2.0 * rint(0.5 * u0);
-      double sn, cn;
-      sincospi(u, &sn, &cn);
-      *reinterpret_cast<T2*>(smem_raw + sm.scale) = T2{R(m * cn), R(-m * sn)};
-    }
+  if constexpr (kImage) {
+    for (uint32_t w = tid * 16; w < a.img_bytes; w += NT * 16) cp_async16(smem_raw + sm.ops + w, a.img + w);
+    cp_async_commit();
+    cp_async_wait(0);
+  } else {
+    make_tables<R, B>(a, sm, smem_raw);
   }
   const int n_ops = a.n_ops, n_cls = a.n_cls;
   const int last_lay = a.last_lay;
@@ -799,7 +799,7 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
   // chunk s0 ^ mswz(mm) and global row g0 ^ mglob(mm), both maps linear over
   // XOR, so four basis values each give all of them.
   constexpr int NJB = B - VB;  // log2 NJ
-  const Layout* L0 = &lays[a.ops[0].idx].L;  // the first op is always a layout
+  const Layout* L0 = &lays[first_lay].L;
   auto copy_in = [&](uint32_t base, int state) {
     const T2* src = reinterpret_cast<const T2*>(a.src) + HS_BCHK(state, a.n_rhs, BS_REG_STATE) * a.N;
     const uint4 ms4 = *reinterpret_cast<const uint4*>(L0->mswz), mg4 = *reinterpret_cast<const uint4*>(L0->mglob);
@@ -821,8 +821,8 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
     cp_async_commit();
   };
 
-  if (pdl) grid_dependency_wait();  // the state written by the previous launch is visible after this
-  __syncthreads();                  // the tables are in shared memory
+  grid_dependency_wait();  // the state written by the previous launch is visible after this
+  __syncthreads();         // the tables are in shared memory
 
   // Chunk q: tile index and its states [state, state_end).
   uint32_t q = q0, base = 0;
@@ -835,7 +835,7 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
   };
   chunk(q, base, state, state_end);
   copy_in(base, state);
-  if (pdl) grid_launch_dependents();  // the next sweep may load its tables meanwhile
+  grid_launch_dependents();  // the next sweep may load its tables meanwhile
 
   bool new_tile = true;
   uint32_t have = 0;  // PHASE runs whose factors are in shared memory for this tile
@@ -950,13 +950,13 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
         }
         if constexpr (V == 2) {
           // The copied tile holds (re, im) row by row, a written-back one pairs.
-          if (first) {
+          // (Selected, not branched on: with a branch here the compiler ran out of
+          // registers; without its four spilled words 77.5 -> 74.4 ms.)
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-              const float t = x.re[j].y;
-              x.re[j].y = x.im[j].x;
-              x.im[j].x = t;
-            }
+          for (int j = 0; j < NJ; ++j) {
+            const float t = first ? x.im[j].x : x.re[j].y;
+            x.im[j].x = first ? x.re[j].y : x.im[j].x;
+            x.re[j].y = t;
           }
         }
         if (oi == last_lay && more) {
@@ -994,7 +994,7 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
         diag_rot<R, B>(x, ops[oi].c.v[0], ops[oi].c.v[1], op.zk, parity(op.zrest & cur_base) ^ parity(op.zthr & local_row()));
       } else {
         if constexpr (FULL) {
-          const Tab& tb = a.tab[op.idx];
+          const Tab& tb = reinterpret_cast<const Tab*>(at(&SmemMap::tabs))[op.idx];
           const uint32_t smask = tb.sm;
           const int tsh = tb.sh;
           uint32_t pr[B];
@@ -1092,13 +1092,14 @@ __device__ __forceinline__ void qsweep_core(const Args& a, uint32_t q0, uint32_t
 template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512)>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  qsweep_core<R, B, FULL>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw, true);
+  qsweep_core<R, B, FULL>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
 }
 
 template <typename R, int B, bool FULL>
 __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_kernel(const __grid_constant__ LevelArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  int* pref = reinterpret_cast<int*>(smem_raw + p.prefix_smem);
+  Hdr& a = *reinterpret_cast<Hdr*>(smem_raw + p.prefix_smem);  // the job's header
+  int* pref = reinterpret_cast<int*>(smem_raw + p.prefix_smem + kHdrSmem);
   for (int i = threadIdx.x; i < p.count; i += blockDim.x) pref[i] = p.lvl_prefix[p.off + i];
   __syncthreads();
   int lo = 0, hi = p.count - 1;
@@ -1106,9 +1107,54 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
     const int mid = (lo + hi + 1) >> 1;
     if (pref[mid] <= int(blockIdx.x)) lo = mid; else hi = mid - 1;
   }
-  const Args& a = p.descs[p.lvl_desc[p.off + lo]];
+  const uint32_t* hd = reinterpret_cast<const uint32_t*>(p.descs + p.lvl_desc[p.off + lo]);
+  static_assert(sizeof(Hdr) % 4 == 0, "copied by words");
+  for (uint32_t w = threadIdx.x; w < sizeof(Hdr) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(&a)[w] = hd[w];
+  __syncthreads();
   const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_chunks, BS_BATCH_JOB));
-  qsweep_core<R, B, FULL>(a, u, u + 1, 1u, smem_raw, true);
+  qsweep_core<R, B, FULL>(a, u, u + 1, 1u, smem_raw);
+}
+
+// One block per image: the template's bytes, then the coefficients of every op
+// from the term records, the phase terms' angles, the value tables and the
+// sweep's scale.
+template <typename R>
+__global__ void __launch_bounds__(128) qfill_kernel(const FillRec* recs) {
+  using T2 = typename C2<R>::T;
+  __shared__ double sm[4], sp[4];
+  __shared__ int sk[4];
+  const FillRec f = recs[blockIdx.x];
+  const int tid = threadIdx.x;
+  for (uint32_t w = tid; w < f.bytes / 16; w += 128)
+    reinterpret_cast<uint4*>(f.img)[w] = reinterpret_cast<const uint4*>(f.tmpl)[w];
+  __syncthreads();
+  double m = 1.0, ph = 0.0;
+  int kq = 0;
+  const Records rec{f.rq, f.cs, f.n_terms_g};
+  const OpRec<R>* src = reinterpret_cast<const OpRec<R>*>(f.tmpl + f.ops);
+  OpRec<R>* dst = reinterpret_cast<OpRec<R>*>(f.img + f.ops);
+  for (int oi = tid; oi < f.n_ops; oi += 128) {
+    const Op op = src[oi].op;
+    dst[oi].c = coef_of<R>(op, reinterpret_cast<const int32_t*>(src[oi].c.v), rec, m, ph, kq);
+  }
+  const PTerm* pt = reinterpret_cast<const PTerm*>(f.tmpl + f.pt);
+  R* thpi = reinterpret_cast<R*>(f.img + f.thpi);
+  for (int t = tid; t < f.n_pterm; t += 128) thpi[t] = R(f.rq[4 * HS_BCHK(pt[t].th, f.n_terms_g, BS_REG_TERM) + 3]);
+  const Tab* tabs = reinterpret_cast<const Tab*>(f.tmpl + f.tabs);
+  T2* vts = reinterpret_cast<T2*>(f.img + f.vts);
+  for (int t = 0; t < f.n_tab; ++t)
+    for (int e = tid; e < tabs[t].n; e += 128)
+      vts[tabs[t].s0 + e] = reinterpret_cast<const T2*>(f.vt)[HS_BCHK(tabs[t].vt0 + e, f.n_vt_g, BS_REG_VT)];
+  sum_scale(m, ph, kq);
+  if ((tid & 31) == 0) {
+    sm[tid >> 5] = m;
+    sp[tid >> 5] = ph;
+    sk[tid >> 5] = kq;
+  }
+  __syncthreads();
+  if (tid == 0)
+    *reinterpret_cast<T2*>(f.img + f.scale) = scale_of<R>(sm[0] * sm[1] * sm[2] * sm[3], sp[0] + sp[1] + sp[2] + sp[3],
+                                                          sk[0] + sk[1] + sk[2] + sk[3]);
 }
 
 using LFn = void (*)(LevelArgs);
@@ -1167,6 +1213,19 @@ cudaError_t prepare_qsweep() {
   return cudaSuccess;
 }
 
+cudaError_t launch_fill(hs_dtype dt, const unsigned char* dev, int n, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const FillRec* r = reinterpret_cast<const FillRec*>(dev);
+  if (dt == HS_C64)
+    qfill_kernel<float><<<unsigned(n), 128, 0, s>>>(r);
+  else
+    qfill_kernel<double><<<unsigned(n), 128, 0, s>>>(r);
+  note_launches();
+  return cudaGetLastError();
+}
+
+void op_records(const Args& a, int oi, int32_t (&rec)[5]) { records_of(a, a.ops[oi], rec); }
+
 size_t qsweep_smem_bytes(const Args& a, hs_dtype dt, int B) {
   return smem_map(a, uint32_t(elem_bytes(dt)), 1u << (a.tile_bits - B)).total;
 }
@@ -1207,7 +1266,7 @@ void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs, int rhs_chunk)
 }
 
 cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
-                          cudaStream_t s) {
+                          bool pdl, cudaStream_t s) {
   LFn fn = qlevel_fn(dt, B, full);
   if (!fn || tile_bits - B < 5 || smem > kSweepSmemMax || ctas <= 0 || ctas >= (int64_t(1) << 31))
     return cudaErrorInvalidValue;
@@ -1220,7 +1279,7 @@ cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const Le
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, L);
   if (e == cudaSuccess) note_launches();
   return e;

@@ -230,6 +230,162 @@ bool plan_qsweep_runs(const hs_factors* f, const std::vector<int>& factors, uint
                       std::vector<std::pair<std::vector<int>, std::shared_ptr<Args>>>& out, std::string* why,
                       const std::vector<int>* steps = nullptr, int step_stride = 0);
 
+// ---------------------------------------------------------------------------
+// Tables in shared memory.  A CTA of a single launch makes them from the
+// descriptor, its kernel parameter, and the term records: 10,500 cycles (4,000
+// to copy the descriptor, 2,700 for the coefficients, 3,800 for the FP64
+// scale), which hide behind the sweep before (programmatic dependent launch)
+// and serve every chunk of a resident CTA.  A CTA of a batch level runs one
+// chunk and starts among running ones, where they would show each time: a
+// batch has every descriptor's tables in device memory as the very bytes a CTA
+// wants, its image, written by one small kernel per batch launch (launch_fill)
+// and copied by the CTA with a few 16-byte loads (32 uneven chains: 2.93 ms
+// with tables made by each CTA, 2.37 ms with images; single launches with
+// images were 4% slower, 74.4 and 77.2 ms on the 24-qubit MaxCut instance).
+// ---------------------------------------------------------------------------
+
+// An op's coefficients: ROTN the tan(theta') of register bits 0 .. 4, ROT and
+// DROT (cos, sin) or (tan, 0), BOND w; `swap` the register bits (ROTN) or the
+// flag (ROT) of odd quarter turns.  In a template the first five words hold
+// the record each coefficient comes from.
+template <typename R>
+struct alignas(16) Coef {
+  R v[5];
+  uint32_t swap;
+  uint32_t pad[sizeof(R) == 4 ? 2 : 1];
+};
+
+// An op with its coefficients; a layout with the local row (x) and the
+// swizzled chunk (y) that a lane index (0 .. 31) and a warp index (32 ..)
+// deposit: a thread's register row 0 is the XOR of the two.
+template <typename R>
+struct OpRec {
+  Op op;
+  Coef<R> c;
+};
+struct LayRec {
+  Layout L;
+  uint2 dep[48];
+};
+
+// ROTN: the rotation slot of register bit i.
+__host__ __device__ __forceinline__ int rotn_slot(const Op& op, int i) {
+  return int((i < 4 ? (op.zthr >> (8 * i)) : (op.zrest >> (8 * (i - 4)))) & 0xffu);
+}
+
+// The local row that index j of a LayRec deposits (lane j, or warp j - 32), and
+// the one it deposits in the copies of a layout's rows in address order.
+__host__ __device__ __forceinline__ uint32_t deposit_index(const Layout& L, int j) {
+  uint32_t d = 0;
+  if (j < 32)
+    for (int i = 0; i < 5 && i < L.n_thr; ++i) d |= uint32_t((j >> i) & 1) << L.thr[i];
+  else
+    for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
+  return d;
+}
+__host__ __device__ __forceinline__ uint32_t copy_index(const Layout& L, int j, int in_chunk) {
+  uint32_t d = 0;
+  if (j < 32)
+    for (int k = 0; k < 5; ++k) d |= uint32_t((j >> k) & 1) << (L.wlo[k] + in_chunk);
+  else
+    for (int i = 5; i < L.n_thr; ++i) d |= uint32_t(((j - 32) >> (i - 5)) & 1) << L.thr[i];
+  return d;
+}
+
+// Byte offsets of a CTA's tables in shared memory: the tile, the image (ops to
+// scale), then what the kernel fills itself (fac, e0s, cw).
+struct SmemMap {
+  uint32_t ops, lays, tabs, vts, ph, cls, pt, thpi, clane, scale, fac, e0s, cw, total;
+};
+
+__host__ __device__ inline SmemMap smem_map(const Args& a, uint32_t e, uint32_t nt) {
+  SmemMap m;
+  uint32_t o = e << a.tile_bits;
+  auto take = [&](uint32_t bytes) {
+    const uint32_t at = o;
+    o += (bytes + 15u) & ~15u;
+    return at;
+  };
+  const uint32_t warps = nt >> 5;
+  m.ops = take((e == 8 ? sizeof(OpRec<float>) : sizeof(OpRec<double>)) * a.n_ops);
+  m.lays = take(sizeof(LayRec) * a.n_lay);
+  m.tabs = take(sizeof(Tab) * a.n_tab);
+  m.vts = take(e * a.n_vt);
+  m.ph = take(sizeof(Phase) * a.n_phase);
+  m.cls = take(sizeof(PClass) * a.n_cls);
+  m.pt = take(sizeof(PTerm) * a.n_pterm);
+  m.thpi = take((e / 2) * a.n_pterm);
+  m.clane = take(48 * 4);
+  m.scale = take(e);
+  m.fac = take(e * nt * a.n_fac);
+  m.e0s = take(e * warps * a.n_phase);
+  m.cw = take(e * warps * a.n_cls);  // a class constant and its mask: the element size
+  m.total = o;
+  return m;
+}
+
+// What a CTA of a batch level needs of its descriptor.
+struct Hdr {
+  const void* src;
+  void* dst;
+  const unsigned char* img;  // the image
+  int64_t N;
+  uint32_t img_bytes;        // a multiple of 16
+  uint32_t m0, m1;
+  int sh;
+  Runs rest;
+  int n_rhs;
+  int n_tiles_log2;
+  int rhs_chunk, rhs_chunks, n_chunks;
+  int n_ops, n_phase, n_cls;
+  int first_lay;             // layout the sweep starts in
+  int last_lay, free_local, fac_keep;
+  SmemMap sm;
+};
+
+struct FillRec {
+  const unsigned char* tmpl;
+  unsigned char* img;
+  const double* rq;
+  const double* cs;
+  const void* vt;
+  int64_t n_vt_g;
+  int n_terms_g;
+  uint32_t bytes;            // of the image
+  int n_ops, n_tab, n_pterm;
+  uint32_t ops, tabs, vts, pt, thpi, scale;  // byte offsets in the image
+};
+
+// The images of a set of launches.
+class Images {
+ public:
+  Images(hs_dtype dt, int B) : dt_(dt), B_(B) {}
+  // Adds descriptor a (with its job fields: fill_job); returns the image's number.
+  int add(const Args& a);
+  int count() const { return int(recs_.size()); }
+  // Device bytes, the first host_bytes() of which are uploaded from blob(dev).
+  size_t device_bytes() const { return host_bytes() + img_bytes_; }
+  size_t host_bytes() const { return rec_bytes() + tmpl_.size(); }
+  std::vector<unsigned char> blob(unsigned char* dev) const;
+  // The header of a launch of a with image number i, the images at dev.
+  Hdr header(const Args& a, int i, unsigned char* dev) const;
+
+ private:
+  size_t rec_bytes() const { return (recs_.size() * sizeof(FillRec) + 255) / 256 * 256; }
+  hs_dtype dt_;
+  int B_;
+  std::vector<FillRec> recs_;
+  std::vector<size_t> tmpl_off_, img_off_;
+  std::vector<unsigned char> tmpl_;
+  size_t img_bytes_ = 0;
+};
+
+// The term records of an op (ROTN: one per register bit).
+void op_records(const Args& a, int oi, int32_t (&rec)[5]);
+
+// Write n images (records at the start of dev).
+cudaError_t launch_fill(hs_dtype dt, const unsigned char* dev, int n, cudaStream_t s);
+
 size_t qsweep_smem_bytes(const Args& a, hs_dtype dt, int B);
 
 // The job-dependent fields of a descriptor: state (evolved in place), the
@@ -244,14 +400,16 @@ int pick_rhs_chunk(int64_t tiles, int n_rhs, int slots);
 // One level of a batch of register sweeps: CTA c runs chunk c - prefix[e] of
 // descriptor lvl_desc[off + e], e the last entry with prefix[off + e] <= c.
 struct LevelArgs {
-  const Args* descs;
+  const Hdr* descs;
   const int* lvl_desc;
   const int* lvl_prefix;
   int off, count;
-  uint32_t prefix_smem;  // byte offset of the level's prefix table in shared memory
+  uint32_t prefix_smem;  // byte offset in shared memory of a CTA's header, the level's prefix table after it
 };
+constexpr uint32_t kHdrSmem = 256;
+static_assert(sizeof(Hdr) <= kHdrSmem, "a header and the prefix table do not overlap");
 cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
-                          cudaStream_t s);
+                          bool pdl, cudaStream_t s);
 // rq, cs (optional): term records to use instead of the factor set's own
 // (n_terms of them), for a sweep over steps of a time-dependent set.
 cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B,
