@@ -190,7 +190,10 @@ int hs_evolve(const hs_factors* f, void* psi, int n_rhs, int n_steps, void* cuda
 
 /* Evolution method selector for hs_evolve_ex. */
 typedef enum {
-  HS_METHOD_AUTO = 0,  /* fused tile sweeps where possible (same as hs_evolve) */
+  HS_METHOD_AUTO = 0,  /* as hs_evolve: the autotuner's choice where there is one; register sweeps (REG)
+                          for sets of single-qubit X, equal-coupling XX + YY + ZZ and diagonal terms
+                          from a measured size on, when no other option is set and every factor fits;
+                          else fused tile sweeps where possible */
   HS_METHOD_PLAIN = 1, /* one row-parallel diagonal-times-vector launch per factor application */
   HS_METHOD_FUSED = 2, /* tile sweeps; factors that do not fit a tile fall back to PLAIN */
   HS_METHOD_REG = 3    /* register-blocked tile sweeps, one state per tile: each thread keeps 2^reg_bits

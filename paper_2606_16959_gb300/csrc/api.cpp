@@ -726,8 +726,11 @@ int hs_plan_schedule(const uint64_t* x, const uint64_t* z, size_t n_terms, int n
   return HS_OK;
 }
 
-// Resolve evolve options: method, tile bits, rhs block, low bits.
-int resolve_opts(const hs_factors* f, int n_rhs, const hs_evolve_opts* opts, hs_evolve_opts& o, int& tb, int& rb) {
+// Resolve evolve options: method, tile bits, rhs block, low bits.  n_steps: the
+// steps of a static evolution (0: a drive schedule, which stays with the staged
+// sweeps unless asked otherwise).
+int resolve_opts(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_opts* opts, hs_evolve_opts& o, int& tb,
+                 int& rb) {
   o = hs_evolve_opts{HS_METHOD_AUTO, 0, 0, 0, 0, 0, 0, 0};
   if (opts) o = *opts;
   if (o.method == HS_METHOD_AUTO && o.tile_bits == 0 && o.rhs_block == 0 && o.low_bits == 0 && o.max_fuse == 0 &&
@@ -736,6 +739,9 @@ int resolve_opts(const hs_factors* f, int n_rhs, const hs_evolve_opts* opts, hs_
     if (hs::tuned_opts(f, n_rhs, &t)) {
       t.use_graph = o.use_graph;
       o = t;
+    } else if (const int qt = n_steps > 0 && o.reg_bits == 0 ? hs::q::auto_tile_bits(f, n_rhs, n_steps) : 0) {
+      o.method = HS_METHOD_REG;
+      o.tile_bits = qt;
     }
   }
   if (o.low_bits <= 0) o.low_bits = min_low_bits(f->dtype);
@@ -779,17 +785,35 @@ int resolve_opts(const hs_factors* f, int n_rhs, const hs_evolve_opts* opts, hs_
   return HS_OK;
 }
 
+// Options and launch schedule of a static evolution.  Register sweeps that the
+// library chose by itself must hold every factor: where one does not fit, the
+// staged sweeps take the whole evolution.
+static int plan_static(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_opts* opts, hs_evolve_opts& o,
+                       int& tb, int& rb, std::vector<hs::Sweep>& sw, QPlans& qp) {
+  int rc = resolve_opts(f, n_rhs, n_steps, opts, o, tb, rb);
+  if (rc != HS_OK || n_steps == 0) return rc;
+  sw = schedule(f, n_steps, o, tb);
+  if (o.method != HS_METHOD_REG) return HS_OK;
+  plan_reg(f, sw, tb, o.reg_bits, qp);
+  if (has_plain(sw) && (!opts || opts->method == HS_METHOD_AUTO) && hs::q::auto_tile_bits(f, n_rhs, n_steps)) {
+    rc = resolve_opts(f, n_rhs, 0, opts, o, tb, rb);
+    if (rc != HS_OK || o.method == HS_METHOD_REG) return rc;  // (REG: the autotuner's choice)
+    qp.clear();
+    sw = schedule(f, n_steps, o, tb);
+  }
+  return HS_OK;
+}
+
 int hs_evolve_plan(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_opts* opts, int* n_sweeps,
                    int* n_plain, int* tile_bits, int* rhs_block) {
   if (!f) return fail(HS_EINVAL, "factors is NULL");
   if (n_rhs < 1 || n_steps < 0) return fail(HS_EINVAL, "n_rhs must be >= 1 and n_steps >= 0");
   hs_evolve_opts o;
   int tb = 0, rb = 0;
-  int rc = resolve_opts(f, n_rhs, opts, o, tb, rb);
-  if (rc != HS_OK) return rc;
-  std::vector<hs::Sweep> sw = schedule(f, n_steps, o, tb);
+  std::vector<hs::Sweep> sw;
   QPlans qp;
-  if (o.method == HS_METHOD_REG) plan_reg(f, sw, tb, o.reg_bits, qp);
+  int rc = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp);
+  if (rc != HS_OK) return rc;
   int ns = 0, np = 0;
   for (const hs::Sweep& w : sw) (w.fused ? ns : np) += 1;
   if (n_sweeps) *n_sweeps = ns;
@@ -808,7 +832,9 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
   if (reinterpret_cast<uintptr_t>(psi) % 16) return fail(HS_EINVAL, "psi must be 16-byte aligned");
   hs_evolve_opts o;
   int tb = 0, rb = 0;
-  int rc0 = resolve_opts(f, n_rhs, opts, o, tb, rb);
+  std::vector<hs::Sweep> sw;
+  QPlans qp;
+  int rc0 = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp);
   if (rc0 != HS_OK) return rc0;
   if (n_steps == 0) return HS_OK;
   {
@@ -817,12 +843,9 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
   const size_t state_bytes = size_t(n_rhs) * size_t(f->plan.N) * hs::elem_bytes(f->dtype);
-  std::vector<hs::Sweep> sw = schedule(f, n_steps, o, tb);
-  QPlans qp;
   if (o.method == HS_METHOD_REG) {
     cudaError_t e = hs::q::prepare_qsweep();
     if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
-    plan_reg(f, sw, tb, o.reg_bits, qp);
   }
   const QPlans* qpp = qp.empty() ? nullptr : &qp;
   const bool scratch_needed = has_plain(sw);
@@ -915,7 +938,7 @@ int hs_evolve_td_plan(const hs_factors* f, int n_rhs, int n_steps, const hs_evol
   if (n_rhs < 1 || n_steps < 0) return fail(HS_EINVAL, "n_rhs must be >= 1 and n_steps >= 0");
   hs_evolve_opts o;
   int tb = 0, rb = 0;
-  int rc = resolve_opts(f, n_rhs, opts, o, tb, rb);
+  int rc = resolve_opts(f, n_rhs, 0, opts, o, tb, rb);
   if (rc != HS_OK) return rc;
   int ns = 0, np = 0;
   if (n_steps > 0) {
@@ -973,7 +996,7 @@ int hs_evolve_td(hs_factors* f, void* psi, int n_rhs, const double* drive, int n
     if (!std::isfinite(drive[k])) return fail(HS_EINVAL, "non-finite drive value at step " + std::to_string(k));
   hs_evolve_opts o;
   int tb = 0, rb = 0;
-  int rc0 = resolve_opts(f, n_rhs, opts, o, tb, rb);
+  int rc0 = resolve_opts(f, n_rhs, 0, opts, o, tb, rb);
   if (rc0 != HS_OK) return rc0;
   if (n_steps == 0) return HS_OK;
   {

@@ -3,6 +3,7 @@
 // layouts between them.
 #include <algorithm>
 #include <map>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -42,7 +43,80 @@ uint32_t pext32(uint32_t v, uint32_t m) {
   return out;
 }
 
+// XX, YY and ZZ of one qubit pair with one coefficient, next to each other in
+// any order from term j on, act as one BOND (static sets: a drive may part the
+// three).
+bool bond_first(const hs_factors* f, const Group& G, int j) {
+  const Plan& p = f->plan;
+  if (f->bin.coeff1 || j < G.first || j + 3 > G.last) return false;
+  const uint64_t u = p.x[j] | p.z[j];
+  int kinds = 0;
+  for (int k = j; k < j + 3; ++k) {
+    if ((p.x[k] | p.z[k]) != u || (p.x[k] & ~u) || p.coeff[k] != p.coeff[j]) return false;
+    if ((p.x[k] && p.x[k] != u) || (p.z[k] && p.z[k] != u)) return false;
+    kinds |= p.x[k] ? (p.z[k] ? 2 : 1) : 4;
+  }
+  return __builtin_popcountll(u) == 2 && kinds == 7;
+}
+
+// Several terms and a value table of at most two slots.
+bool has_small_table(const Group& G) {
+  return G.last - G.first > 1 && G.vt0 >= 0 && G.nslot >= 1 && G.nslot <= 2 && G.vt_n <= kMaxVt;
+}
+
 }  // namespace
+
+// The least work (states x rows) at which register sweeps are the library's
+// choice, by measurement against the staged sweeps (us for ten first-order
+// steps, staged / register):
+//   complex128, 15 x 3 states (3 * 2^15 rows): Heisenberg 648 / 411, TFIM 578 /
+//     492; 14 x 5 MaxCut 431 / 475; 17 x 1: 455 / 443 and 782 / 520; 18 x 1
+//     MaxCut 869 / 523; 20 x 4 11800 / 5400.  A fourth-order step has ten
+//     different exponentials to plan: two steps of 17 x 1 Heisenberg 832 / 902.
+//   complex64 bonds, 18 x 4 376 / 258, 20 x 1 792 / 257; 18 x 1 with two bonds
+//     to a factor 163 / 197, hence the line above that size.
+// A staged sweep re-reads its tile from shared memory for every factor; below
+// these sizes that fits the time the register sweep's tables take to make.
+// Tiles of 2^10 rows (2^11 from 2^20 rows on) give complex128 enough CTAs: 18 x
+// 1 Heisenberg takes 491, 533 and 744 us with 10, 11 and 12 bits.  complex64:
+// 12 bits, 13 from 2^22 rows on (22 x 1 Heisenberg: 585 and 549 us).
+// The sets: X on one qubit, equal-coupling bonds and diagonal terms (a set with
+// unequal XX and YY takes two rotations a bond and is up to twice as slow as
+// the staged sweeps; three-qubit flips need plain launches), at least half as
+// many flips and at most twice as many diagonal terms as qubits (a diagonal
+// Hamiltonian is one stored factor: 41 / 78).
+int auto_tile_bits(const hs_factors* f, int n_rhs, int n_steps) {
+  const Plan& p = f->plan;
+  const int n = p.n_qubits;
+  const bool c64 = f->dtype == HS_C64;
+  if (f->bin.coeff1 || n < 13 || n > 30 || n_steps > 4096) return 0;
+  int flips = 0, bonds = 0, diag = 0;
+  std::set<int> seen;  // (a higher-order formula applies the same terms in several factors)
+  for (const Group& G : p.groups) {
+    if (!seen.insert(G.first).second) continue;
+    if (!(G.last - G.first == 3 && bond_first(f, G, G.first)) && has_small_table(G)) return 0;
+    for (int j = G.first; j < G.last; ++j) {
+      if (bond_first(f, G, j)) {
+        ++bonds;
+        j += 2;
+      } else if (p.x[j] == 0) {
+        ++diag;
+      } else if (__builtin_popcountll(p.x[j]) == 1 && p.z[j] == 0) {
+        ++flips;
+      } else {
+        return 0;
+      }
+    }
+  }
+  if (2 * (flips + bonds) < n || diag > 2 * n) return 0;
+  const int64_t rows = int64_t(n_rhs) << n;
+  if (c64) {
+    if (flips || rows < (int64_t(1) << 20)) return 0;
+    return rows >= (int64_t(1) << 22) ? 13 : 12;
+  }
+  if (rows < (p.order > 2 ? int64_t(1) << 18 : int64_t(3) << 15)) return 0;
+  return rows >= (int64_t(1) << 20) ? 11 : 10;
+}
 
 bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
                  Args& a, std::string* why, const std::vector<int>* steps, int step_stride) {
@@ -87,23 +161,11 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
     const size_t first_op = ops.size();
     const Group& G = p.groups[g];
     if ((G.span & ~uint64_t(local_mask)) != 0) return fail("factor flips outside the tile");
-    // XX, YY and ZZ of one qubit pair with one coefficient, next to each other
-    // in any order, act as one BOND (static sets: a drive may part the three).
-    auto bond_at = [&](int j) {
-      if (steps || f->bin.coeff1 || j < G.first || j + 3 > G.last) return false;
-      const uint64_t u = p.x[j] | p.z[j];
-      int kinds = 0;
-      for (int k = j; k < j + 3; ++k) {
-        if ((p.x[k] | p.z[k]) != u || (p.x[k] & ~u) || p.coeff[k] != p.coeff[j]) return false;
-        if ((p.x[k] && p.x[k] != u) || (p.z[k] && p.z[k] != u)) return false;
-        kinds |= p.x[k] ? (p.z[k] ? 2 : 1) : 4;
-      }
-      return __builtin_popcountll(u) == 2 && kinds == 7;
-    };
+    auto bond_at = [&](int j) { return !steps && bond_first(f, G, j); };
     // A factor of several terms with a value table of at most two slots (a
     // bond whose couplings differ) is read from its table; a single term is
     // cheaper as its rotation, and three equal ones as a BOND.
-    if (!(G.last - G.first == 3 && bond_at(G.first)) && G.last - G.first > 1 && G.vt0 >= 0 && G.nslot >= 1 && G.nslot <= 2 && G.vt_n <= kMaxVt) {
+    if (!(G.last - G.first == 3 && bond_at(G.first)) && has_small_table(G)) {
       const uint32_t u = G.nslot == 2 ? p.slot_u[G.slot0 + 1] : 0u;
       if (__builtin_popcount(loc(u)) <= 2) {
         // (value tables hold one step's values: not in a sweep that spans steps)

@@ -223,7 +223,11 @@ __host__ __device__ __forceinline__ uint32_t across_patterns(uint32_t mu_mask) {
 bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
                  Args& a, std::string* why, const std::vector<int>* steps = nullptr, int step_stride = 0);
 
-// The same for a run of factors that may exceed a descriptor's limits: the
+// The tile bits with which HS_METHOD_AUTO takes register sweeps, 0 where it
+// takes the staged ones.
+int auto_tile_bits(const hs_factors* f, int n_rhs, int n_steps);
+
+// plan_qsweep for a run of factors that may exceed a descriptor's limits: the
 // run is split into consecutive shorter runs (same local mask) until each
 // fits.  Returns false if a single factor cannot be expressed.
 bool plan_qsweep_runs(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,

@@ -1,0 +1,106 @@
+"""HS_METHOD_AUTO's choice between staged and register sweeps against the staged sweeps.
+
+The staged sweeps apply the factors in the formula's order; the register sweeps compute the same
+product with exact rotations.  Tolerances: complex128 1e-12 and complex64 2e-6 sqrt(steps x
+exponentials) relative (each application rounds an amplitude a few times at 1.1e-16 / 6e-8).
+"""
+import numpy as np
+import pytest
+
+from paper_2606_16959_gb300 import hs, workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2606_16959_gb300 import _build
+    _build.build()
+    hs.lib()
+
+
+def _bond(n, a, b, w):
+    return [(W.label_of(n, {a: p, b: p}), w) for p in "XYZ"]
+
+
+def _terms(kind, n):
+    rng = np.random.default_rng(n)
+    t = []
+    if kind == "chain":
+        for a in range(n):
+            t += _bond(n, a, (a + 1) % n, rng.uniform(0.5, 1.5))
+    elif kind == "far":  # bonds no tile of 2^10 rows holds: the staged sweeps take the set
+        for a in range(n - 1):
+            t += _bond(n, a, a + 1, 0.7)
+        t += _bond(n, n // 2 + 1, n - 1, 0.4) + _bond(n, 0, n // 2, 0.3)
+    elif kind in ("field", "mixed"):  # flips and three-qubit diagonal terms, in descending order
+        for a in range(n - 1, -1, -1):
+            t.append((W.label_of(n, {a: "X"}), rng.uniform(-1, 1)))
+            t.append((W.label_of(n, {a: "Z", (a + 3) % n: "Z", (a + 5) % n: "Z"}), rng.uniform(-1, 1)))
+        if kind == "field":  # (interleaved, each factor is read from a small table: staged)
+            t = t[::2] + t[1::2]
+    elif kind == "tfim":
+        h = W.tfim_chain(n, 1.1, 0.7)
+        t = list(zip(h.labels, h.coeffs))
+    elif kind == "unequal":
+        for a in range(n - 1):
+            t += [(W.label_of(n, {a: p, a + 1: p}), w) for p, w in zip("XYZ", (0.9, 0.9, 0.5))]
+    elif kind == "diagonal":
+        t = [(W.label_of(n, {a: "Z", (a + 1) % n: "Z"}), 0.3) for a in range(n)]
+    return [l for l, _ in t], np.array([c for _, c in t])
+
+
+# (terms, qubits, states, dtype, order, steps, takes register sweeps)
+CASES = [
+    ("chain", 15, 3, "c128", 2, 4, True), ("chain", 15, 2, "c128", 1, 4, False),
+    ("chain", 13, 12, "c128", 1, 3, True), ("chain", 12, 32, "c128", 1, 3, False),
+    ("chain", 18, 1, "c128", 4, 2, True), ("chain", 17, 1, "c128", 4, 2, False),
+    ("chain", 20, 1, "c64", 1, 4, True), ("chain", 19, 1, "c64", 1, 4, False),
+    ("chain", 20, 5, "c64", 2, 2, True), ("chain", 20, 2, "c128", 1, 2, True),
+    ("tfim", 16, 2, "c128", 1, 5, True), ("field", 17, 1, "c128", 2, 3, True),
+    ("mixed", 17, 1, "c128", 2, 3, False),
+    ("tfim", 20, 1, "c64", 1, 4, False), ("far", 18, 1, "c128", 1, 2, None), ("far", 24, 1, "c64", 1, 1, None),
+    ("unequal", 18, 1, "c128", 1, 2, False), ("diagonal", 18, 1, "c128", 1, 2, False),
+]
+
+
+@pytest.mark.parametrize("kind,n,rhs,dt,order,steps,reg", CASES)
+def test_auto_matches_staged(kind, n, rhs, dt, order, steps, reg):
+    labels, c = _terms(kind, n)
+    f = hs.hs_build_factors(labels, c, 1.0, 20, 4, dt, order=order)
+    tdt = torch.complex64 if dt == "c64" else torch.complex128
+    g = torch.Generator(device="cuda").manual_seed(n)
+    psi = torch.randn(rhs, 1 << n, dtype=tdt, device="cuda", generator=g)
+    psi /= torch.linalg.vector_norm(psi, dim=1, keepdim=True)
+    a, b = psi.clone(), psi.clone()
+    pa = hs.hs_evolve_plan(f, rhs, steps)
+    pr = hs.hs_evolve_plan(f, rhs, steps, method=hs.HS_METHOD_FUSED)
+    hs.hs_evolve(f, a, steps)
+    hs.hs_evolve_ex(f, b, steps, method=hs.HS_METHOD_FUSED)
+    if reg:
+        r = psi.clone()
+        hs.hs_evolve_ex(f, r, steps, method=hs.HS_METHOD_REG, tile_bits=pa[2])
+        assert torch.equal(a, r) and not torch.equal(a, b)
+    elif reg is not None:
+        assert pa == pr and torch.equal(a, b)
+    k = steps * {1: 1, 2: 2, 4: 10}[order]
+    tol = 2e-6 * np.sqrt(k) if dt == "c64" else 1e-12
+    d = torch.linalg.vector_norm((a - b).to(torch.complex128), dim=1)
+    assert float(d.max()) <= tol
+    if reg:  # as a graph and under a caller's capture
+        assert pa[1] == 0
+        e = psi.clone()
+        hs.hs_evolve_ex(f, e, steps, use_graph=True)
+        assert torch.equal(a, e)
+        e.copy_(psi)
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        gr = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(gr, stream=s):
+            hs.hs_evolve(f, e, steps)
+        gr.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(a, e)
