@@ -1461,7 +1461,9 @@ int hs_expectation(const hs_dia* a, const void* psi, int n_rhs, void* cuda_strea
     if (e == cudaSuccess) e = out.alloc(size_t(n_rhs) * sizeof(double4), s);
     if (e != cudaSuccess) return cuda_err(e, "expectation buffers");
     if (sym) {
-      const int rb = n_rhs >= 4 ? 4 : (n_rhs >= 2 ? 2 : 1);
+      // Few rows want the parallelism of one state per thread (whole call, 12
+      // qubits, four complex128 states: 67 us with four, general kernel 61).
+      const int rb = n_rhs >= 4 && a->N > (1 << 16) ? 4 : (n_rhs >= 2 && a->N > (1 << 15) ? 2 : 1);
       if (a->dtype == HS_C64)
         launch_expect_sym<float2>(a, psi, n_rhs, rb, nb, part.as<double4>(), s);
       else
