@@ -786,21 +786,32 @@ int resolve_opts(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_op
 }
 
 // Options and launch schedule of a static evolution.  Register sweeps that the
-// library chose by itself must hold every factor: where one does not fit, the
-// staged sweeps take the whole evolution.
+// library chose by itself (`own`) must hold every factor: where one does not
+// fit, the staged sweeps take the whole evolution.
 static int plan_static(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_opts* opts, hs_evolve_opts& o,
-                       int& tb, int& rb, std::vector<hs::Sweep>& sw, QPlans& qp) {
+                       int& tb, int& rb, std::vector<hs::Sweep>& sw, QPlans& qp, bool& own) {
+  own = false;
   int rc = resolve_opts(f, n_rhs, n_steps, opts, o, tb, rb);
   if (rc != HS_OK || n_steps == 0) return rc;
   sw = schedule(f, n_steps, o, tb);
   if (o.method != HS_METHOD_REG) return HS_OK;
   plan_reg(f, sw, tb, o.reg_bits, qp);
-  if (has_plain(sw) && (!opts || opts->method == HS_METHOD_AUTO) && hs::q::auto_tile_bits(f, n_rhs, n_steps)) {
-    rc = resolve_opts(f, n_rhs, 0, opts, o, tb, rb);
-    if (rc != HS_OK || o.method == HS_METHOD_REG) return rc;  // (REG: the autotuner's choice)
+  hs_evolve_opts o0;
+  int tb0 = 0, rb0 = 0;
+  rc = resolve_opts(f, n_rhs, 0, opts, o0, tb0, rb0);
+  own = rc == HS_OK && o0.method != HS_METHOD_REG;  // (else the caller's or the autotuner's choice)
+  if (!own) return rc;
+  if (has_plain(sw)) {
+    own = false;
+    o = o0;
+    tb = tb0;
+    rb = rb0;
     qp.clear();
     sw = schedule(f, n_steps, o, tb);
+    return HS_OK;
   }
+  for (auto& a : qp)
+    if (a) a->exact_scale = f->dtype == HS_C64;
   return HS_OK;
 }
 
@@ -812,7 +823,8 @@ int hs_evolve_plan(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_
   int tb = 0, rb = 0;
   std::vector<hs::Sweep> sw;
   QPlans qp;
-  int rc = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp);
+  bool own;
+  int rc = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp, own);
   if (rc != HS_OK) return rc;
   int ns = 0, np = 0;
   for (const hs::Sweep& w : sw) (w.fused ? ns : np) += 1;
@@ -834,7 +846,8 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
   int tb = 0, rb = 0;
   std::vector<hs::Sweep> sw;
   QPlans qp;
-  int rc0 = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp);
+  bool own;
+  int rc0 = plan_static(f, n_rhs, n_steps, opts, o, tb, rb, sw, qp, own);
   if (rc0 != HS_OK) return rc0;
   if (n_steps == 0) return HS_OK;
   {
@@ -856,7 +869,7 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
   }
 
   if (o.use_graph) {
-    hs_factors::GraphKey key{psi, n_rhs, n_steps, int(o.method) * 128 + o.max_fuse + 16384 * o.reg_bits,
+    hs_factors::GraphKey key{psi, n_rhs, n_steps, int(o.method) * 128 + o.max_fuse + 16384 * o.reg_bits + (own ? 1 << 20 : 0),
                              tb + 64 * o.smem_kb, (rb * 64 + o.low_bits) * 2 + (o.no_tables != 0), nullptr, 0};
     cudaGraphExec_t exec = nullptr;
     {

@@ -666,13 +666,17 @@ __device__ __forceinline__ void sum_scale(double& m, double& ph, int& kq) {
   }
 }
 
+// The sweep's scale rounded to R; lost: what the rounding took off.
 template <typename R>
-__device__ __forceinline__ typename C2<R>::T scale_of(double m, double ph, int kq) {
+__device__ __forceinline__ typename C2<R>::T scale_of(double m, double ph, int kq,
+                                                      typename C2<R>::T* lost = nullptr) {
   using T2 = typename C2<R>::T;
   const double u0 = ph + 0.5 * double(kq & 3), u = u0 - 2.0 * rint(0.5 * u0);
   double sn, cn;
   sincospi(u, &sn, &cn);
-  return T2{R(m * cn), R(-m * sn)};
+  const T2 c{R(m * cn), R(-m * sn)};
+  if (lost) *lost = T2{R(m * cn - double(c.x)), R(-m * sn - double(c.y))};
+  return c;
 }
 
 // The records of op oi of a descriptor.
@@ -736,7 +740,10 @@ __device__ __forceinline__ void make_tables(const Args& a, const SmemMap& sm, un
       ops[oi].c = coef_of<R>(op, rec, t, m, ph, kq);
     }
     sum_scale(m, ph, kq);
-    if (tid == 0) *reinterpret_cast<T2*>(smem_raw + sm.scale) = scale_of<R>(m, ph, kq);
+    if (tid == 0) {
+      T2* out = reinterpret_cast<T2*>(smem_raw + sm.scale);
+      out[0] = scale_of<R>(m, ph, kq, sizeof(T2) == 8 && a.exact_scale ? out + 1 : nullptr);
+    }
   }
 }
 
@@ -753,7 +760,7 @@ __device__ __forceinline__ void make_tables(const Args& a, const SmemMap& sm, un
 // the current one finishes in registers and goes straight back to HBM.
 // ---------------------------------------------------------------------------
 // D: Args (the tables are made here) or Hdr (they are copied from the image).
-template <typename R, int B, bool FULL, typename D>
+template <typename R, int B, bool FULL, bool EXACT, typename D>
 __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1, uint32_t stride,
                                             unsigned char* smem_raw) {
   using T2 = typename C2<R>::T;
@@ -1013,11 +1020,22 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
     if (out_scale.y != R(0)) {
       if constexpr (V == 2) {
         const float2 c = dup(out_scale.x), s = dup(out_scale.y), ns = dup(-out_scale.y);
+        if constexpr (EXACT) {
+          const float2 lost = reinterpret_cast<const float2*>(at(&SmemMap::scale))[1];
+          const float2 cl = dup(lost.x), sl = dup(lost.y), nsl = dup(-lost.y);
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          const float2 r = x.re[j], m = x.im[j];
-          x.re[j] = fma2(r, c, __fmul2_rn(m, ns));
-          x.im[j] = fma2(r, s, __fmul2_rn(m, c));
+          for (int j = 0; j < NJ; ++j) {
+            const float2 r = x.re[j], m = x.im[j];
+            x.re[j] = fma2(r, c, fma2(m, ns, fma2(r, cl, __fmul2_rn(m, nsl))));
+            x.im[j] = fma2(r, s, fma2(m, c, fma2(r, sl, __fmul2_rn(m, cl))));
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) {
+            const float2 r = x.re[j], m = x.im[j];
+            x.re[j] = fma2(r, c, __fmul2_rn(m, ns));
+            x.im[j] = fma2(r, s, __fmul2_rn(m, c));
+          }
         }
       } else {
 #pragma unroll
@@ -1088,11 +1106,14 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
 // FULL: the kernel with the TAB and general-rotation paths; sweeps without
 // them run the lighter instantiation.  NT: threads per CTA the instantiation
 // is built for (2^(tile_bits - B); 512 for 2^14-row complex64 tiles with five
-// register bits, one CTA per SM).
-template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512)>
+// register bits, one CTA per SM).  EXACT: a bond sweep applies its scale to more
+// than R's precision.  Rounded, a scale shifts the norm by up to 6e-8 a sweep, all
+// one way: 1.1e-5 over 200 steps of a 20-qubit Heisenberg chain, 1e-8 with it.  (An
+// instantiation of its own: as a branch it cost the MaxCut sweeps 0.5%.)
+template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = false>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  qsweep_core<R, B, FULL>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
+  qsweep_core<R, B, FULL, EXACT>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
 }
 
 template <typename R, int B, bool FULL>
@@ -1112,7 +1133,7 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
   for (uint32_t w = threadIdx.x; w < sizeof(Hdr) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(&a)[w] = hd[w];
   __syncthreads();
   const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_chunks, BS_BATCH_JOB));
-  qsweep_core<R, B, FULL>(a, u, u + 1, 1u, smem_raw);
+  qsweep_core<R, B, FULL, false>(a, u, u + 1, 1u, smem_raw);
 }
 
 // One block per image: the template's bytes, then the coefficients of every op
@@ -1173,7 +1194,9 @@ QFn qsweep_fn_t(hs_dtype dt, int B, int tile_bits) {
   if (B == 4 && tb <= 9) return dt == HS_C64 ? qsweep_kernel<float, 4, FULL> : qsweep_kernel<double, 4, FULL>;
   return nullptr;
 }
-QFn qsweep_fn(hs_dtype dt, int B, bool full, int tile_bits) {
+QFn qsweep_fn(hs_dtype dt, int B, bool full, int tile_bits, bool exact = false) {
+  if (exact && !full && dt == HS_C64 && B == 5 && tile_bits >= 10 && tile_bits <= 13)
+    return qsweep_kernel<float, 5, false, 256, true>;
   return full ? qsweep_fn_t<true>(dt, B, tile_bits) : qsweep_fn_t<false>(dt, B, tile_bits);
 }
 
@@ -1203,6 +1226,9 @@ cudaError_t prepare_qsweep() {
                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
       if (e == cudaSuccess && v == 0)
         e = cudaFuncSetAttribute((const void*)qsweep_fn(dts[v], Bs[v], full, 14),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
+      if (e == cudaSuccess && v == 0)
+        e = cudaFuncSetAttribute((const void*)qsweep_fn(dts[v], Bs[v], full, 13, true),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void*)qlevel_fn(dts[v], Bs[v], full),
@@ -1288,7 +1314,7 @@ cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const Le
 cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B, bool pdl,
                           cudaStream_t s, const double* rq, const double* cs, int n_terms) {
   const Plan& p = f->plan;
-  QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits);
+  QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits, a.exact_scale != 0);
   if (!fn || a.tile_bits - B < 5 || a.tile_bits > p.n_qubits) return cudaErrorInvalidValue;
   const size_t smem = qsweep_smem_bytes(a, f->dtype, B);
   if (smem > kSweepSmemMax) return cudaErrorInvalidValue;

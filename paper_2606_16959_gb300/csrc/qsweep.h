@@ -161,6 +161,7 @@ struct Args {
                      // 0: the runs share slots and their factors are computed on each use
   int last_lay;      // index of the last LAYOUT op
   int free_local;    // 1: the last layout's warp bits are the first one's
+  int exact_scale;   // complex64 bonds: 1 takes the instantiation that applies the scale unrounded
   int full;          // 1 if a TAB op or a rotation other than tan form occurs (the larger kernel)
   Op ops[kMaxOps];
   Layout lay[kMaxLayouts];
@@ -320,7 +321,7 @@ __host__ __device__ inline SmemMap smem_map(const Args& a, uint32_t e, uint32_t 
   m.pt = take(sizeof(PTerm) * a.n_pterm);
   m.thpi = take((e / 2) * a.n_pterm);
   m.clane = take(48 * 4);
-  m.scale = take(e);
+  m.scale = take(16);  // complex64: the scale and what its rounding lost
   m.fac = take(e * nt * a.n_fac);
   m.e0s = take(e * warps * a.n_phase);
   m.cw = take(e * warps * a.n_cls);  // a class constant and its mask: the element size

@@ -78,16 +78,18 @@ def test_auto_matches_staged(kind, n, rhs, dt, order, steps, reg):
     a, b = psi.clone(), psi.clone()
     pa = hs.hs_evolve_plan(f, rhs, steps)
     pr = hs.hs_evolve_plan(f, rhs, steps, method=hs.HS_METHOD_FUSED)
+    k = steps * {1: 1, 2: 2, 4: 10}[order]
+    tol = 2e-6 * np.sqrt(k) if dt == "c64" else 1e-12
     hs.hs_evolve(f, a, steps)
     hs.hs_evolve_ex(f, b, steps, method=hs.HS_METHOD_FUSED)
     if reg:
         r = psi.clone()
         hs.hs_evolve_ex(f, r, steps, method=hs.HS_METHOD_REG, tile_bits=pa[2])
-        assert torch.equal(a, r) and not torch.equal(a, b)
+        assert not torch.equal(a, b)
+        # (complex64: REG asked for rounds a sweep's scale, the library's choice does not)
+        assert torch.equal(a, r) if dt == "c128" else float(torch.linalg.vector_norm(a - r)) <= tol
     elif reg is not None:
         assert pa == pr and torch.equal(a, b)
-    k = steps * {1: 1, 2: 2, 4: 10}[order]
-    tol = 2e-6 * np.sqrt(k) if dt == "c64" else 1e-12
     d = torch.linalg.vector_norm((a - b).to(torch.complex128), dim=1)
     assert float(d.max()) <= tol
     if reg:  # as a graph and under a caller's capture
