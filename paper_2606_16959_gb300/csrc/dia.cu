@@ -45,6 +45,13 @@ struct hs_dia {
   void* d_vals = nullptr;
   int64_t* d_meta = nullptr;   // [offs(D), rowbase(D)]
   int device = 0;
+  // The XOR masks i ^ c of all entries (i, c) that can differ from zero, sorted
+  // (H of Pauli terms: the terms' flips; products: the pairwise XORs); empty if
+  // nothing is known.
+  std::vector<uint32_t> flips;
+  // Slot table of the evolution by masks (see make_slots), or null: [u(W),
+  // first(W), row bases].
+  int32_t* d_slots = nullptr;
   bool real_symmetric = false; // known real and equal to its transpose (H of terms with even numbers of Y)
 };
 
@@ -59,6 +66,7 @@ using hs::report_error;
 
 constexpr int kThreads = 256;               // elements per task block
 constexpr int64_t kAlignElems = 8;          // 128 B for complex128, 64 B for complex64
+constexpr size_t kMaxFlips = 4096;           // XOR masks of a matrix the library keeps track of
 constexpr int kMaxCandidates = 65536;       // structural diagonals of H from terms
 constexpr double kDropRel = 1.0 / 70368744177664.0;  // 2^-46
 
@@ -440,6 +448,178 @@ __global__ void __launch_bounds__(32 * W) spmv_kernel(const typename CT<R>::T2* 
   }
 }
 
+// ---------------------------------------------------------------------------
+// Evolution by slots.  A product of Pauli sums has one entry per row and flip
+// mask u, in column i ^ u, but the mask's entries are spread over 2^|u|
+// diagonals: a two-term TFIM propagator on 16 qubits stores 455 diagonals for
+// 137 masks, and seven stored values in ten are zero.  The evolution first
+// gathers them (slot-major: slots[k N + i] = A(i, i ^ u_k)), then every step
+// reads a third of the bytes (72 MB, which the L2 keeps, not 239 MB from HBM at
+// 4.7 TB/s), all 16-byte loads: rows i and i + 1 of complex64 have their columns
+// in one aligned pair.  64 complex64 steps of that propagator: 3.25 -> 0.81 ms;
+// of one with three flips (697 masks): 22.0 -> 4.6 ms.
+// ---------------------------------------------------------------------------
+constexpr size_t kMaxSlotRows = size_t(1) << 17;
+constexpr int32_t kNoDiag = INT32_MIN;
+constexpr size_t kMaxSlotBytes = size_t(4) << 30;
+template <typename T2>
+__device__ __forceinline__ bool not_finite(T2 v) {
+  return !(isfinite(v.x) && isfinite(v.y));
+}
+
+// slots from the diagonals; flag[0] = 1 if psi (np amplitudes) has a value that is not finite.
+template <typename T2>
+__global__ void __launch_bounds__(kThreads) slots_kernel(const int32_t* __restrict__ tab, int W, int log2n,
+                                                         const T2* __restrict__ vals, int64_t n_vals, T2* __restrict__ slots,
+                                                         const T2* __restrict__ psi, int64_t np, uint32_t* flag) {
+  const int64_t step = int64_t(gridDim.x) * kThreads, first = int64_t(blockIdx.x) * kThreads + threadIdx.x;
+  const int64_t N = int64_t(1) << log2n;
+  for (int64_t e = first; e < int64_t(W) << log2n; e += step) {
+    const int k = int(e >> log2n);
+    const int64_t i = e & (N - 1);
+    uint32_t p = 0, j = 0;
+    for (uint32_t m = uint32_t(__ldg(tab + k)); m; m &= m - 1u, ++j) p |= ((uint32_t(i) >> (__ffs(m) - 1)) & 1u) << j;
+    const int32_t b = __ldg(tab + 2 * W + __ldg(tab + W + k) + int(p));
+    T2 v;
+    v.x = v.y = 0;
+    if (b != kNoDiag) v = vals[HS_BCHK(int64_t(b) + i, n_vals, hs::BS_DIA_VAL)];
+    slots[e] = v;
+  }
+  bool bad = false;
+  for (int64_t e = first; e < np; e += step) bad = bad || not_finite(psi[e]);
+  if (bad) *flag = 1u;
+}
+
+// Two rows of complex64 or one of complex128: 16 bytes.
+template <typename R>
+struct Quad;
+template <>
+struct Quad<float> {
+  static constexpr int V = 2;
+  float4 q;
+  __device__ __forceinline__ float2 get(int e) const { return e ? make_float2(q.z, q.w) : make_float2(q.x, q.y); }
+};
+template <>
+struct Quad<double> {
+  static constexpr int V = 1;
+  double2 q;
+  __device__ __forceinline__ double2 get(int) const { return q; }
+};
+
+// y = A x for n_rhs states, W warps as G slices of the slots by W / G slices of
+// the tile's rows.  flag[0] set: a value of x is not finite, and A's stored zeros
+// count (0 times infinity), so the rows are summed from the diagonals; flag[1] is
+// set when a value of y is not.
+template <typename R, int RB, int W, int G>
+__global__ void __launch_bounds__(32 * W) slot_spmv_kernel(const int32_t* __restrict__ tab, int n_slots,
+                                                           const typename CT<R>::T2* __restrict__ slots,
+                                                           const typename CT<R>::T2* __restrict__ vals,
+                                                           const int64_t* __restrict__ meta, int D,
+                                                           const typename CT<R>::T2* __restrict__ x,
+                                                           typename CT<R>::T2* __restrict__ y, int64_t N, int n_rhs,
+                                                           int64_t n_vals, uint32_t* flag) {
+  using T2 = typename CT<R>::T2;
+  using Q = Quad<R>;
+  constexpr int V = Q::V, TILE = 32 * (W / G) * V;
+  __shared__ T2 part[G - 1][RB][TILE];
+  __shared__ uint32_t us[kMaxFlips];
+  for (int k = threadIdx.x; k < n_slots; k += 32 * W) us[k] = uint32_t(tab[k]);
+  __syncthreads();
+  pdl_wait();
+  pdl_trigger();
+  const bool general = *reinterpret_cast<volatile uint32_t*>(flag) != 0u;
+  const int wid = int(threadIdx.x) >> 5;
+  const int g = wid / (W / G), row = ((wid % (W / G)) * 32 + (int(threadIdx.x) & 31)) * V;
+  bool bad = false;
+  for (int64_t tile = blockIdx.x; tile * TILE < N; tile += gridDim.x) {
+    const int64_t i0 = tile * TILE + row;
+    for (int r0 = 0; r0 < n_rhs; r0 += RB) {
+      R ax[V][RB], ay[V][RB];
+#pragma unroll
+      for (int e = 0; e < V; ++e)
+#pragma unroll
+        for (int q = 0; q < RB; ++q) ax[e][q] = ay[e][q] = R(0);
+      if (i0 < N && !general) {
+        const Q* sl = reinterpret_cast<const Q*>(slots + i0);
+#pragma unroll 4
+        for (int k = g; k < n_slots; k += G) {
+          const uint32_t u = us[k];
+          const Q v = sl[int64_t(k) * (N / V)];
+          const int64_t c = (i0 ^ int64_t(u)) & ~int64_t(V - 1);
+          const bool odd = V == 2 && (u & 1u);
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            if (r0 + q < n_rhs) {
+              const Q w = *reinterpret_cast<const Q*>(x + HS_BCHK(int64_t(r0 + q) * N + c, int64_t(n_rhs) * N, hs::BS_DIA_X));
+#pragma unroll
+              for (int e = 0; e < V; ++e) {
+                const T2 a = v.get(e), b = odd ? w.get(V - 1 - e) : w.get(e);
+                ax[e][q] = fma(a.x, b.x, fma(-a.y, b.y, ax[e][q]));
+                ay[e][q] = fma(a.x, b.y, fma(a.y, b.x, ay[e][q]));
+              }
+            }
+          }
+        }
+      } else if (i0 < N) {
+        for (int k = g; k < D; k += G) {
+          const int64_t d = meta[k], base = meta[D + k];
+          for (int e = 0; e < V; ++e) {
+            const int64_t i = i0 + e, c = i + d;
+            if (uint64_t(c) >= uint64_t(N)) continue;
+            const T2 a = vals[HS_BCHK(base + i, n_vals, hs::BS_DIA_VAL)];
+#pragma unroll
+            for (int q = 0; q < RB; ++q)
+              if (r0 + q < n_rhs) {
+                const T2 b = x[HS_BCHK(int64_t(r0 + q) * N + c, int64_t(n_rhs) * N, hs::BS_DIA_X)];
+                R sx = fma(a.x, b.x, -a.y * b.y), sy = fma(a.x, b.y, a.y * b.x);
+#pragma unroll
+                for (int f = 0; f < V; ++f)
+                  if (f == e) {
+                    ax[f][q] += sx;
+                    ay[f][q] += sy;
+                  }
+              }
+          }
+        }
+      }
+      if (g > 0) {
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            T2 o;
+            o.x = ax[e][q];
+            o.y = ay[e][q];
+            part[g - 1][q][row + e] = o;
+          }
+      }
+      __syncthreads();
+      if (g == 0 && i0 < N) {
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            if (r0 + q < n_rhs) {
+              T2 o;
+              o.x = ax[e][q];
+              o.y = ay[e][q];
+#pragma unroll
+              for (int s2 = 0; s2 < G - 1; ++s2) {
+                const T2 v = part[s2][q][row + e];
+                o.x += v.x;
+                o.y += v.y;
+              }
+              bad = bad || not_finite(o);
+              y[int64_t(r0 + q) * N + i0 + e] = o;
+            }
+          }
+      }
+      __syncthreads();
+    }
+  }
+  if (bad) flag[1] = 1u;
+}
+
 // Expectation values: block b of state r sums conj(psi_i) (A psi)_i and |psi_i|^2
 // over a grid-stride set of rows in FP64; partial[r * gridDim.x + b] gets the
 // block sums (re, im, norm, unused).
@@ -666,6 +846,7 @@ void destroy(hs_dia* m) {
   cudaDeviceSynchronize();
   if (m->d_vals) cudaFree(m->d_vals);
   if (m->d_meta) cudaFree(m->d_meta);
+  if (m->d_slots) cudaFree(m->d_slots);
   if (cur != m->device) cudaSetDevice(cur);
   delete m;
 }
@@ -674,6 +855,7 @@ void destroy_async(hs_dia* m, cudaStream_t s) {
   if (!m) return;
   if (m->d_vals) cudaFreeAsync(m->d_vals, s);
   if (m->d_meta) cudaFreeAsync(m->d_meta, s);
+  if (m->d_slots) cudaFreeAsync(m->d_slots, s);
   delete m;
 }
 
@@ -733,6 +915,37 @@ int make_dia(int n_qubits, const std::vector<int64_t>& offs, hs_dtype dt, cudaSt
   }
   out = std::move(m);
   return HS_OK;
+}
+
+// The masks of a product and of a sum; empty (unknown) if either is or beyond
+// kMaxFlips.
+std::vector<uint32_t> tidy_flips(std::vector<uint32_t> f) {
+  std::sort(f.begin(), f.end());
+  f.erase(std::unique(f.begin(), f.end()), f.end());
+  if (f.size() > kMaxFlips) f.clear();
+  return f;
+}
+std::vector<uint32_t> flips_mul(const hs_dia* a, const hs_dia* b) {
+  std::vector<uint32_t> f;
+  if (a->n_qubits <= 20) {
+    std::vector<uint8_t> has(size_t(a->N), 0);
+    for (uint32_t u : a->flips)
+      for (uint32_t v : b->flips) has[u ^ v] = 1;
+    for (uint32_t u = 0; u < has.size(); ++u)
+      if (has[u]) f.push_back(u);
+    if (f.size() > kMaxFlips) f.clear();
+    return f;
+  }
+  f.reserve(a->flips.size() * b->flips.size());
+  for (uint32_t u : a->flips)
+    for (uint32_t v : b->flips) f.push_back(u ^ v);
+  return tidy_flips(std::move(f));
+}
+std::vector<uint32_t> flips_add(const hs_dia* a, const hs_dia* b) {
+  if (a->flips.empty() || b->flips.empty()) return {};
+  std::vector<uint32_t> f = a->flips;
+  f.insert(f.end(), b->flips.begin(), b->flips.end());
+  return tidy_flips(std::move(f));
 }
 
 // Task table: one (diagonal, first element) per `per` elements; block0[k]
@@ -828,6 +1041,7 @@ int combine(const hs_dia* a, const hs_dia* b, const std::vector<int64_t>& offs, 
   hs::note_launches();
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "combine launch");
+  if (!b) m->flips = a->flips;
   out = std::move(m);
   return HS_OK;
 }
@@ -887,6 +1101,7 @@ int add_dia(const hs_dia* a, const hs_dia* b, cudaStream_t s, DiaPtr& out) {
   hs::note_launches();
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "add launch");
+  m->flips = flips_add(a, b);
   out = std::move(m);
   return HS_OK;
 }
@@ -899,6 +1114,7 @@ int identity_dia(int n_qubits, cudaStream_t s, DiaPtr& out) {
   hs::note_launches();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "identity");
+  m->flips = {0u};
   out = std::move(m);
   return HS_OK;
 }
@@ -974,6 +1190,7 @@ int spgemm_impl(const hs_dia* A, const hs_dia* B, double alpha, cudaStream_t s, 
       nnz += st[k].nz;
     }
   if (fro) *fro = std::sqrt(s2);
+  if (std::isfinite(s2)) C->flips = flips_mul(A, B);  // (0 times a value that is not finite is not 0)
   if (keep.size() == offs.size()) {
     C->nnz = nnz;
     out = std::move(C);
@@ -1097,6 +1314,79 @@ cudaError_t launch_spmv(const hs_dia* a, const void* x, void* y, int n_rhs, cuda
   }
   if (n_rhs >= 2) return launch_spmv_w<double, 2>(a, x, y, n_rhs, cfg);
   return launch_spmv_w<double, 1>(a, x, y, n_rhs, cfg);
+}
+
+// The slot table of a matrix whose masks are known, where that at least halves
+// what an evolution reads (made with the matrix: the evolution can be captured).
+int make_slots(hs_dia* a, cudaStream_t s) {
+  const size_t W = a->flips.size();
+  if (W < 2 || 2 * W > a->offs.size() || a->N < 64 || a->total > INT32_MAX ||
+      W * size_t(a->N) * esize(a->dtype) > kMaxSlotBytes)
+    return HS_OK;
+  std::vector<std::pair<int64_t, int>> at(a->offs.size());
+  for (size_t k = 0; k < at.size(); ++k) at[k] = {a->offs[k], int(k)};
+  std::sort(at.begin(), at.end());
+  std::vector<int32_t> t(2 * W);
+  for (size_t k = 0; k < W; ++k) {
+    const uint32_t u = a->flips[k];
+    const int c = __builtin_popcount(u);
+    if (c > 12 || t.size() - 2 * W + (size_t(1) << c) > kMaxSlotRows) return HS_OK;
+    t[k] = int32_t(u);
+    t[W + k] = int32_t(t.size() - 2 * W);
+    for (uint32_t p = 0; p < (1u << c); ++p) {
+      int64_t d = 0;  // (i ^ u) - i: a set bit is taken off, a clear one added
+      int j = 0;
+      for (uint32_t m = u; m; m &= m - 1u, ++j) d += ((p >> j) & 1u) ? -int64_t(m & (0u - m)) : int64_t(m & (0u - m));
+      const auto it = std::lower_bound(at.begin(), at.end(), std::make_pair(d, 0));
+      const bool has = it != at.end() && it->first == d;
+      t.push_back(has ? int32_t(a->start[size_t(it->second)] + std::min<int64_t>(0, d)) : kNoDiag);
+    }
+  }
+  cudaError_t e = pool_malloc(reinterpret_cast<void**>(&a->d_slots), t.size() * sizeof(int32_t), s);
+  if (e != cudaSuccess) {
+    a->d_slots = nullptr;
+    return cuda_err(e, "cudaMallocAsync(slot table)");
+  }
+  e = cudaMemcpyAsync(a->d_slots, t.data(), t.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+  return e == cudaSuccess ? HS_OK : cuda_err(e, "slot table upload");
+}
+
+template <typename R, int RB, int W, int G>
+cudaError_t launch_slot_spmv_k(const hs_dia* a, const void* slots, const void* x, void* y, int n_rhs,
+                               uint32_t* flag, cudaLaunchConfig_t& cfg) {
+  using T2 = typename CT<R>::T2;
+  constexpr int TILE = 32 * (W / G) * Quad<R>::V;
+  const int64_t tiles = (a->N + TILE - 1) / TILE;
+  cfg.gridDim = dim3(unsigned(std::min<int64_t>(tiles, hs::kSMs * (64 / W))), 1u, 1u);
+  cfg.blockDim = dim3(32 * W, 1u, 1u);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, slot_spmv_kernel<R, RB, W, G>, (const int32_t*)a->d_slots,
+                                           int(a->flips.size()), (const T2*)slots,
+                                           (const T2*)a->d_vals, (const int64_t*)a->d_meta, int(a->offs.size()),
+                                           (const T2*)x, (T2*)y, a->N, n_rhs, a->total, flag);
+  if (e == cudaSuccess) hs::note_launches();
+  return e;
+}
+
+// Slices (warps by slot slices) measured on two- and three-flip TFIM propagators
+// of 10 to 16 qubits: one state 16 by 16 (64 steps, three flips, 16 qubits,
+// complex64: 4.65 ms; 16 by 8 6.2, 16 by 4 5.2, 32 by 8 6.2), several states
+// fewer slices (four states: 16 by 4 5.0 ms for 32 steps, 16 by 16 5.4).
+cudaError_t launch_slot_spmv(const hs_dia* a, const void* slots, const void* x, void* y, int n_rhs,
+                             uint32_t* flag, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (a->dtype == HS_C64) {
+    if (n_rhs >= 4) return launch_slot_spmv_k<float, 4, 16, 4>(a, slots, x, y, n_rhs, flag, cfg);
+    if (n_rhs >= 2) return launch_slot_spmv_k<float, 2, 16, 8>(a, slots, x, y, n_rhs, flag, cfg);
+    return launch_slot_spmv_k<float, 1, 16, 16>(a, slots, x, y, n_rhs, flag, cfg);
+  }
+  if (n_rhs >= 2) return launch_slot_spmv_k<double, 2, 8, 4>(a, slots, x, y, n_rhs, flag, cfg);
+  return launch_slot_spmv_k<double, 1, 16, 16>(a, slots, x, y, n_rhs, flag, cfg);
 }
 
 template <typename T2>
@@ -1246,6 +1536,7 @@ int hs_dia_from_masks(const uint64_t* x, const uint64_t* z, const double* coeffs
   H->nnz = nnz;
   // i^y is real for an even number of Y, and entries (i, c) and (c, i) are then
   // the same sum: parity(z & i) = parity(z & c) for every term that flips i into c.
+  if (n_qubits <= 32) H->flips = tidy_flips(std::vector<uint32_t>(masks.begin(), masks.end()));
   H->real_symmetric = true;
   for (int y : ty) H->real_symmetric = H->real_symmetric && (y & 1) == 0;
   e = cudaStreamSynchronize(s);
@@ -1349,6 +1640,7 @@ int hs_spme(const hs_dia* a, double t, double tol, int max_iter, void* cuda_stre
   int k = 0;
   bool ok = false;
   rc = spme_impl(a, t, tol, max_iter, 0, s, U, &k, &ok);
+  if (rc == HS_OK) rc = make_slots(U.get(), s);
   if (rc) return rc;
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_err(e, "spme");
@@ -1519,8 +1811,35 @@ int hs_dia_evolve(const hs_dia* u, void* psi, int n_rhs, int n_steps, void* cuda
   if (e != cudaSuccess) return cuda_err(e, "cudaMallocAsync(scratch state)");
   void* a = psi;
   void* b = tmp.p;
+  // By slots where the masks are known and half the diagonals or fewer; the
+  // gather costs about one step.
+  DevBuf slots, flags;
+  const int W = int(u->flips.size());
+  bool by_slots = n_steps >= 4 && u->d_slots;
+  if (by_slots) {
+    const size_t sb = size_t(W) * size_t(u->N) * esize(u->dtype);
+    by_slots = slots.alloc(sb, s) == cudaSuccess &&
+               flags.alloc((size_t(n_steps) + 1) * sizeof(uint32_t), s) == cudaSuccess;
+    if (!by_slots) cudaGetLastError();  // no room: from the diagonals
+  }
+  if (by_slots) {
+    e = cudaMemsetAsync(flags.p, 0, (size_t(n_steps) + 1) * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return cuda_err(e, "evolve flags");
+    const int64_t np = int64_t(n_rhs) * u->N, work = std::max(np, int64_t(W) * u->N);
+    const unsigned grid = unsigned(std::min<int64_t>((work + kThreads - 1) / kThreads, hs::kSMs * 32));
+    if (u->dtype == HS_C64)
+      slots_kernel<float2><<<grid, kThreads, 0, s>>>(u->d_slots, W, u->n_qubits, (const float2*)u->d_vals, u->total, slots.as<float2>(),
+                                                     (const float2*)psi, np, flags.as<uint32_t>());
+    else
+      slots_kernel<double2><<<grid, kThreads, 0, s>>>(u->d_slots, W, u->n_qubits, (const double2*)u->d_vals, u->total, slots.as<double2>(),
+                                                      (const double2*)psi, np, flags.as<uint32_t>());
+    hs::note_launches();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_err(e, "evolve layout launch");
+  }
   for (int k = 0; k < n_steps; ++k) {
-    e = launch_spmv(u, a, b, n_rhs, s, k > 0);
+    e = by_slots ? launch_slot_spmv(u, slots.p, a, b, n_rhs, flags.as<uint32_t>() + k, s)
+                 : launch_spmv(u, a, b, n_rhs, s, k > 0);
     if (e != cudaSuccess) return cuda_err(e, "evolve launch");
     std::swap(a, b);
   }
@@ -1544,6 +1863,8 @@ int hs_dia_convert(const hs_dia* a, hs_dtype dtype, void* cuda_stream, hs_dia** 
   rc = combine(a, nullptr, a->offs, ka, kb, make_double2(1.0, 0.0), make_double2(0.0, 0.0), dtype, s, m);
   if (rc) return rc;
   m->real_symmetric = a->real_symmetric;
+  if (a->d_slots) rc = make_slots(m.get(), s);
+  if (rc) return rc;
   *out = m.release();
   return HS_OK;
 }
