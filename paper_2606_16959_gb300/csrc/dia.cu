@@ -52,6 +52,7 @@ struct hs_dia {
   // Slot table of the evolution by masks (see make_slots), or null: [u(W),
   // first(W), row bases].
   int32_t* d_slots = nullptr;
+  bool finite = false;         // every value is known to be finite
   bool real_symmetric = false; // known real and equal to its transpose (H of terms with even numbers of Y)
 };
 
@@ -97,6 +98,12 @@ __device__ __forceinline__ double2 ld(const float2* p, int64_t i) {
 __device__ __forceinline__ void st(double2* p, int64_t i, double2 v) { p[i] = v; }
 __device__ __forceinline__ void st(float2* p, int64_t i, double2 v) {
   p[i] = make_float2(__double2float_rn(v.x), __double2float_rn(v.y));
+}
+
+// v != 0 without the FP64 pipe (a comparison there costs as much as a
+// multiply-add).
+__device__ __forceinline__ bool nonzero(double v) {
+  return ((unsigned(__double2hiint(v)) << 1) | unsigned(__double2loint(v))) != 0u;
 }
 
 struct Stat {
@@ -242,6 +249,12 @@ struct GemmArgs {
 constexpr int kGemmEPT = 4;
 constexpr int kPairChunk = 256;
 
+// SKIP (all values finite): a product with a stored zero is left out, which
+// changes no sum.  The FP64 pipe bounds the kernel (four multiply-adds a product
+// at 1.7 per clock and SM), and in a product of Pauli sums most factors are
+// zeros, above bit 5 for whole warps.  (Step search and exponential of a
+// 12-qubit TFIM chain: 3.20 -> 3.05 ms.)
+template <bool SKIP>
 __global__ void __launch_bounds__(kThreads) gemm_kernel(GemmArgs a) {
   __shared__ Pair sp[kPairChunk];
   const int2 tk = a.task[blockIdx.x];
@@ -270,6 +283,7 @@ __global__ void __launch_bounds__(kThreads) gemm_kernel(GemmArgs a) {
       for (int e = 0; e < kGemmEPT; ++e) {
         if (live[e] && row[e] >= pr.lo && row[e] < pr.hi) {
           const double2 x = a.A[pr.a_rb + row[e]], y = a.B[pr.b_rb + row[e]];
+          if (SKIP && !((nonzero(x.x) || nonzero(x.y)) && (nonzero(y.x) || nonzero(y.y)))) continue;
           acc[e].x = fma(x.x, y.x, fma(-x.y, y.y, acc[e].x));
           acc[e].y = fma(x.x, y.y, fma(x.y, y.x, acc[e].y));
         }
@@ -671,12 +685,6 @@ __global__ void __launch_bounds__(kThreads) expect_kernel(const T2* __restrict__
   }
 }
 
-// v != 0 without the FP64 pipe (a comparison there costs as much as a
-// multiply-add).
-__device__ __forceinline__ bool nonzero(double v) {
-  return ((unsigned(__double2hiint(v)) << 1) | unsigned(__double2loint(v))) != 0u;
-}
-
 // The same for a real symmetric A, RB states at a time: Re <psi|A|psi> = sum_i
 // a_ii |psi_i|^2 + 2 sum_{d > 0} sum_i a_{i, i+d} Re(conj(psi_i) psi_{i+d}), and
 // no imaginary part.  The FP64 pipe bounds the general kernel (96% busy on a
@@ -1042,6 +1050,8 @@ int combine(const hs_dia* a, const hs_dia* b, const std::vector<int64_t>& offs, 
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "combine launch");
   if (!b) m->flips = a->flips;
+  m->finite = !b && a->finite && out_dt == HS_C128 && std::isfinite(alpha_a.x) && std::isfinite(alpha_a.y) &&
+              std::max(std::fabs(alpha_a.x), std::fabs(alpha_a.y)) <= 1.0;
   out = std::move(m);
   return HS_OK;
 }
@@ -1115,6 +1125,7 @@ int identity_dia(int n_qubits, cudaStream_t s, DiaPtr& out) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "identity");
   m->flips = {0u};
+  m->finite = true;
   out = std::move(m);
   return HS_OK;
 }
@@ -1170,7 +1181,10 @@ int spgemm_impl(const hs_dia* A, const hs_dia* B, double alpha, cudaStream_t s, 
   GemmArgs g{(const double2*)A->d_vals, (const double2*)B->d_vals, (double2*)C->d_vals, tabs.offs.as<int64_t>(),
              tabs.start.as<int64_t>(), d_p0.as<int>(), d_pairs.as<Pair>(), d_task.as<int2>(), N, alpha,
              d_part.as<Stat>()};
-  gemm_kernel<<<unsigned(task.size()), kThreads, 0, s>>>(g);
+  if (A->finite && B->finite)
+    gemm_kernel<true><<<unsigned(task.size()), kThreads, 0, s>>>(g);
+  else
+    gemm_kernel<false><<<unsigned(task.size()), kThreads, 0, s>>>(g);
   hs::note_launches();
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_err(e, "spgemm launch");
@@ -1190,7 +1204,8 @@ int spgemm_impl(const hs_dia* A, const hs_dia* B, double alpha, cudaStream_t s, 
       nnz += st[k].nz;
     }
   if (fro) *fro = std::sqrt(s2);
-  if (std::isfinite(s2)) C->flips = flips_mul(A, B);  // (0 times a value that is not finite is not 0)
+  C->finite = std::isfinite(s2);
+  if (C->finite) C->flips = flips_mul(A, B);  // (0 times a value that is not finite is not 0)
   if (keep.size() == offs.size()) {
     C->nnz = nnz;
     out = std::move(C);
@@ -1536,6 +1551,9 @@ int hs_dia_from_masks(const uint64_t* x, const uint64_t* z, const double* coeffs
   H->nnz = nnz;
   // i^y is real for an even number of Y, and entries (i, c) and (c, i) are then
   // the same sum: parity(z & i) = parity(z & c) for every term that flips i into c.
+  double s2 = 0.0;
+  for (const Stat& v : st) s2 += v.s2;
+  H->finite = std::isfinite(s2);
   if (n_qubits <= 32) H->flips = tidy_flips(std::vector<uint32_t>(masks.begin(), masks.end()));
   H->real_symmetric = true;
   for (int y : ty) H->real_symmetric = H->real_symmetric && (y & 1) == 0;
