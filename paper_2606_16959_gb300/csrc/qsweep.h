@@ -66,7 +66,8 @@ struct Op {
   uint8_t type;
   uint8_t ku;     // ROT, TAB, BOND: the flip in register coordinates (TAB: 0 for a one-slot factor)
   uint8_t zk;     // ROT: the register coordinates of z's bits in the tile
-  uint8_t flags;  // ROT: bit 0 = fast path (y = 0 and z = 0); bits 1-2 = q with -i i^y = i^q
+  uint8_t flags;  // ROT: bit 0 = fast path (y = 0 and z = 0); bits 1-2 = q with -i i^y = i^q;
+                  // BOND: 1 = the factor's only terms (it has a value table)
   int16_t idx;    // ROT: rotation slot; TAB: table slot; BOND: bond slot; PHASE: phase slot; LAYOUT: layout slot
   int16_t pad;
   uint32_t zthr;  // ROT: z's bits in the tile on thread positions (local-index mask)
