@@ -87,13 +87,18 @@ int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* 
   const uint64_t all = (1ull << p.n_qubits) - 1;
   for (size_t wi = 0; wi < sw.size(); ++wi) {
     const hs::Sweep& w = sw[wi];
+    // A sweep reads its tables (term records, value tables, factor values) before
+    // it waits for the launch before it.  The first launch waits for all of that
+    // one: it may be the build, or the records or the drive's rebuild, that writes
+    // them.  From the second on every CTA of the launch before has done so.
+    const bool early = wi > 0;
     cudaError_t e;
     if (qp && (*qp)[wi] && rec) {
       const int st = w.steps.empty() ? 0 : w.steps[0];
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, true, s, rec->rq + size_t(4) * st * rec->stride,
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, early, s, rec->rq + size_t(4) * st * rec->stride,
                                rec->cs + size_t(2) * st * rec->stride, (rec->n_steps - st) * rec->stride);
     } else if (qp && (*qp)[wi]) {
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, true, s);
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, early, s);
     } else if (w.fused) {
       hs::SweepLaunch L;
       L.src = cur;
@@ -106,7 +111,7 @@ int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* 
       L.n_factors = int(w.factors.size());
       for (int i = 0; i < L.n_factors; ++i) L.factors[i] = w.factors[i];
       L.smem_budget = smem_budget;
-      L.pdl = true;
+      L.pdl = early;
       L.value_tables = value_tables;
       e = hs::launch_sweep(f, L, s);
     } else {

@@ -302,6 +302,7 @@ int enqueue_batch(hs_batch* b, cudaStream_t s) {
   }
   LevelFn fn = b->dtype == HS_C64 ? level_fn<float>(b->rows) : level_fn<double>(b->rows);
   if (!fn) return hs::report_error(HS_EINVAL, "internal: no batch kernel for this tile size");
+  bool early = false;  // (the factor values are complete before the first level reads them)
   for (const hs_batch::Level& L : b->levels) {
     LevelArgs a{b->d_jobs, b->d_sweeps, b->d_facs, b->d_lvl_sweep, b->d_lvl_prefix, L.off, L.count, b->tile_bits,
                 b->tiles_per_cta};
@@ -314,7 +315,8 @@ int enqueue_batch(hs_batch* b, cudaStream_t s) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
+    early = true;
     cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
     if (e != cudaSuccess) return hs::report_error(HS_ECUDA, std::string("batch level launch: ") + cudaGetErrorString(e));
     hs::note_launches();
