@@ -178,6 +178,19 @@ int hs_plan_schedule(const uint64_t* x, const uint64_t* z, size_t n_terms, int n
                      hs_dtype dtype, int n_steps, int tile_bits, int low_bits, int max_fuse, int commuting,
                      int* n_apps, int* n_sweeps, int* app_factor, int* app_step, int* sweep_of, int capacity);
 
+/* Host-only plan of an evolution by register sweeps (no GPU): the launches of
+ * hs_evolve_ex with HS_METHOD_REG, tile_bits and reg_bits (0: the defaults; up
+ * to the limits there), or with driven != 0 those of hs_evolve_td when its
+ * sweeps span steps.  reserve: shared memory of a CTA that something else takes
+ * (a batch's header and prefix table).  *n_sweeps register sweeps, *n_plain
+ * launches of factors that have no register form, *smem_max the most shared
+ * memory of a sweep's CTA in bytes (at most 232,448 - reserve), *n_lean the
+ * sweeps whose tables fit in their smaller form only, *ops_max the most ops of
+ * a sweep.  Pointers may be NULL.  Errors: HS_EINVAL, HS_EDTYPE. */
+int hs_plan_register(const uint64_t* x, const uint64_t* z, const double* coeffs, size_t n_terms, int n_qubits,
+                     int diag_budget, int order, hs_dtype dtype, int n_steps, int tile_bits, int reg_bits, int driven,
+                     size_t reserve, int* n_sweeps, int* n_plain, int64_t* smem_max, int* n_lean, int* ops_max);
+
 /* Evolve psi in place by n_steps Trotter steps: for each step, apply the
  * factors F_0, ..., F_{G-1} in order (Alg. 3's loop, x <- U x, with U the
  * ordered product of the grouped factors).  psi: device buffer of n_rhs

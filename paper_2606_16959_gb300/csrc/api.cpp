@@ -151,8 +151,9 @@ bool has_plain(const std::vector<hs::Sweep>& sw) {
 // step_stride > 0: the sweeps span steps of a time-dependent set whose term
 // records are kept per step (step_stride records each); a planned sweep's
 // steps become one entry, the step its records start at.
+// reserve: see hs::q::plan_qsweep.
 void plan_reg(const hs_factors* f, std::vector<hs::Sweep>& sw, int tile_bits, int reg_bits, QPlans& qp,
-              int step_stride = 0) {
+              int step_stride = 0, size_t reserve = 0) {
   using Pieces = std::vector<std::pair<std::vector<int>, std::shared_ptr<hs::q::Args>>>;
   std::map<std::tuple<uint32_t, std::vector<int>, std::vector<int>>, std::pair<bool, Pieces>> memo;
   std::vector<hs::Sweep> out;
@@ -172,7 +173,7 @@ void plan_reg(const hs_factors* f, std::vector<hs::Sweep>& sw, int tile_bits, in
       Pieces pieces;
       std::string why;
       const bool ok = hs::q::plan_qsweep_runs(f, w.factors, w.local_mask, tile_bits, reg_bits, pieces, &why,
-                                               step_stride > 0 ? &rel : nullptr, step_stride);
+                                               step_stride > 0 ? &rel : nullptr, step_stride, reserve);
       it = memo.emplace(key, std::make_pair(ok, std::move(pieces))).first;
     }
     if (it->second.first) {
@@ -787,6 +788,47 @@ int resolve_opts(const hs_factors* f, int n_rhs, int n_steps, const hs_evolve_op
   if (o.method != HS_METHOD_PLAIN && tb > hs::max_tile_bits(f->dtype, rb, fused_dmax(f), hs::kSweepSmemMax))
     return fail(HS_EINVAL, "tile_bits exceeds the shared-memory tile for this rhs_block");
   if (tb < 1) return fail(HS_EINVAL, "tile_bits must be >= 1");
+  return HS_OK;
+}
+
+int hs_plan_register(const uint64_t* x, const uint64_t* z, const double* coeffs, size_t n_terms, int n_qubits,
+                     int diag_budget, int order, hs_dtype dtype, int n_steps, int tile_bits, int reg_bits, int driven,
+                     size_t reserve, int* n_sweeps, int* n_plain, int64_t* smem_max, int* n_lean, int* ops_max) {
+  if (!x || !z || !coeffs) return fail(HS_EINVAL, "null argument");
+  if (!valid_dtype(dtype)) return fail(HS_EDTYPE, "dtype must be HS_C64 or HS_C128");
+  if (n_steps < 1 || n_steps > 65535) return fail(HS_EINVAL, "n_steps must be 1..65535");
+  if (reserve > hs::kSweepSmemMax) return fail(HS_EINVAL, "reserve exceeds a CTA's shared memory");
+  hs_factors f;
+  f.dtype = dtype;
+  std::string err;
+  int rc = hs::make_plan(x, z, coeffs, n_terms, n_qubits, diag_budget, dtype, f.plan, &err, order);
+  if (rc != HS_OK) return fail(rc, err);
+  if (driven) f.bin.coeff1 = coeffs;  // (planning looks whether there are any)
+  hs_evolve_opts o{HS_METHOD_REG, tile_bits, 0, 0, 0, 0, 0, 0, reg_bits}, r;
+  int tb = 0, rb = 0;
+  rc = resolve_opts(&f, 1, 0, &o, r, tb, rb);
+  if (rc != HS_OK) return rc;
+  if (r.method != HS_METHOD_REG) return fail(HS_EINVAL, "the state is too small for register sweeps");
+  std::vector<hs::Sweep> sw = schedule(&f, n_steps, r, tb);
+  QPlans qp;
+  plan_reg(&f, sw, tb, r.reg_bits, qp, driven ? int(f.plan.x.size()) * f.plan.n_kinds : 0, reserve);
+  int ns = 0, np = 0, nl = 0, ops = 0;
+  int64_t most = 0;
+  for (const auto& a : qp) {
+    if (!a) {
+      ++np;
+      continue;
+    }
+    ++ns;
+    nl += a->lean;
+    ops = std::max(ops, a->n_ops);
+    most = std::max(most, int64_t(hs::q::qsweep_smem_bytes(*a, dtype, r.reg_bits)));
+  }
+  if (n_sweeps) *n_sweeps = ns;
+  if (n_plain) *n_plain = np;
+  if (smem_max) *smem_max = most;
+  if (n_lean) *n_lean = nl;
+  if (ops_max) *ops_max = ops;
   return HS_OK;
 }
 

@@ -185,6 +185,7 @@ struct hs_batch {
     int off, count;
     int64_t ctas;
     bool full = false;  // register sweeps: some descriptor of the level needs the full kernel
+    bool lean = false;  // some descriptor has its tables in the lean form
   };
   std::vector<Level> levels;
   int max_count = 0;
@@ -293,7 +294,7 @@ int enqueue_batch(hs_batch* b, cudaStream_t s) {
     for (const hs_batch::QGroup& g : b->qgroups)
       for (const hs_batch::Level& L : g.levels) {
         hs::q::LevelArgs a{b->d_qdescs, g.d_lvl_desc, g.d_lvl_prefix, L.off, L.count, uint32_t(g.prefix_smem)};
-        cudaError_t e = hs::q::launch_qlevel(b->dtype, b->reg_bits, L.full, g.tile_bits, a, L.ctas, g.smem, early, s);
+        cudaError_t e = hs::q::launch_qlevel(b->dtype, b->reg_bits, L.full, L.lean, g.tile_bits, a, L.ctas, g.smem, early, s);
         early = true;
         if (e != cudaSuccess)
           return hs::report_error(HS_ECUDA, std::string("batch level launch: ") + cudaGetErrorString(e));
@@ -357,6 +358,16 @@ int create_reg_batch(const hs_batch_job* jobs, size_t n_jobs, const hs_batch_opt
     if (J.n_rhs < 1 || J.n_steps < 0) return hs::report_error(HS_EINVAL, "job " + std::to_string(j) + ": bad n_rhs/n_steps");
     if (reinterpret_cast<uintptr_t>(J.psi) % 16) return hs::report_error(HS_EINVAL, "psi must be 16-byte aligned");
   }
+  // Beside a descriptor's tables a CTA holds its header and the level's prefix
+  // table, one entry per job of the tile size at most.
+  std::map<int, size_t> beside;
+  for (size_t j = 0; j < n_jobs; ++j)
+    if (jobs[j].n_steps > 0) beside[std::min(T, jobs[j].factors->plan.n_qubits)] += sizeof(int);
+  for (auto& kv : beside) {
+    kv.second += hs::q::kHdrSmem + 16;  // (aligned)
+    if (kv.first >= B + 5 && kv.second + (hs::elem_bytes(dt) << kv.first) > hs::kSweepSmemMax)
+      return hs::report_error(HS_EINVAL, "batch needs more shared memory than a CTA has");
+  }
   // Per job (independent, planned on host threads): its sweeps as descriptor
   // pieces (a sweep seen before reuses its pieces), the order in which its
   // levels use them, or "separate" when some sweep has no register form.
@@ -389,7 +400,8 @@ int create_reg_batch(const hs_batch_job* jobs, size_t n_jobs, const hs_batch_opt
       }
       std::vector<std::pair<std::vector<int>, std::shared_ptr<hs::q::Args>>> pieces;
       std::string why;
-      if (!hs::q::plan_qsweep_runs(J.factors, sw[k].factors, sw[k].local_mask, P.Tj, B, pieces, &why)) {
+      if (!hs::q::plan_qsweep_runs(J.factors, sw[k].factors, sw[k].local_mask, P.Tj, B, pieces, &why, nullptr, 0,
+                                    beside.at(P.Tj))) {
         ok = false;
         break;
       }
@@ -452,6 +464,7 @@ int create_reg_batch(const hs_batch_job* jobs, size_t n_jobs, const hs_batch_opt
         g.lvl_desc.push_back(gj.descs[k]);
         g.lvl_prefix.push_back(int(L.ctas));
         L.full = L.full || b->qdescs[gj.descs[k]].full != 0;
+        L.lean = L.lean || b->qdescs[gj.descs[k]].lean != 0;
         L.ctas += gj.units;
         ++L.count;
       }

@@ -124,7 +124,7 @@ int auto_tile_bits(const hs_factors* f, int n_rhs, int n_steps) {
 }
 
 bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
-                 Args& a, std::string* why, const std::vector<int>* steps, int step_stride) {
+                 Args& a, std::string* why, const std::vector<int>* steps, int step_stride, size_t reserve) {
   const Plan& p = f->plan;
   const int n = p.n_qubits;
   const int m = int(p.x.size());
@@ -526,24 +526,36 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
   for (int i = 0; i < a.n_ops; ++i)
     if (a.ops[i].type == OP_LAYOUT) a.last_lay = i;  // the tile buffer's last reader
   a.free_local = warp_pos.front() == warp_pos.back() ? 1 : 0;
-  // Factor slots: every phase its own while that leaves the tile's CTAs per SM
-  // (two with 64 KiB tiles), else shared ones.
+  // Where the phase factors and class constants are kept, the first of these that
+  // leaves two CTAs per SM (64 KiB tiles), else the first that fits: slots of its
+  // own for every phase, shared ones, factors in local memory with one copy of the
+  // class constants (lean).  (A diagonal run of 128 classes in a 128 KiB tile takes
+  // 236,480 bytes with shared slots, 140,240 lean; 300 terms on 20 qubits,
+  // complex128, ten steps in 64 KiB tiles: 2.88 ms with one CTA per SM and shared
+  // slots, 2.67 lean.)
   const uint32_t eb = uint32_t(elem_bytes(f->dtype));
-  a.fac_keep = 1;
-  int n_shared = 0;
+  int n_own = 0, n_shared = 0, own0[kMaxPhase];
   for (int i = 0; i < a.n_phase; ++i) {
     const uint32_t mm = a.ph[i].mu_mask;
     const int own = 1 + B + __builtin_popcount(B == 5 ? inside_patterns<5>(mm) : inside_patterns<4>(mm));
     const int across = __builtin_popcount(B == 5 ? across_patterns<5>(mm) : across_patterns<4>(mm));
-    a.ph[i].fac0 = int16_t(a.n_fac);
-    a.n_fac += own + across;
+    own0[i] = n_own;
+    n_own += own + across;
     n_shared = std::max(n_shared, own + (across ? 1 : 0));
   }
-  if (qsweep_smem_bytes(a, f->dtype, B) > ((size_t(eb) << T) <= (size_t(64) << 10) ? kSweepSmemDefault : kSweepSmemMax)) {
-    a.fac_keep = 0;
-    a.n_fac = n_shared;
-    for (int i = 0; i < a.n_phase; ++i) a.ph[i].fac0 = 0;
-  }
+  auto fits = [&](int form, size_t most) {
+    a.fac_keep = form == 0;
+    a.lean = form == 2;
+    a.n_fac = form == 0 ? n_own : (form == 1 ? n_shared : 0);
+    for (int i = 0; i < a.n_phase; ++i) a.ph[i].fac0 = int16_t(form == 0 ? own0[i] : 0);
+    const size_t bytes = qsweep_smem_bytes(a, f->dtype, B);
+    return bytes <= most && bytes + reserve <= kSweepSmemMax;
+  };
+  const bool small = (size_t(eb) << T) <= (size_t(64) << 10);
+  bool ok = false;
+  for (int form = 0; !ok && form < 3; ++form) ok = fits(form, small ? kSweepSmemDefault : kSweepSmemMax);
+  for (int form = 1; !ok && form < 3; ++form) ok = fits(form, kSweepSmemMax);
+  if (!ok) return fail("the sweep's tables exceed the shared memory of a CTA");
   a.full = 0;
   for (int i = 0; i < a.n_ops; ++i)
     if (a.ops[i].type == OP_TAB || (a.ops[i].type == OP_ROT && !(a.ops[i].flags & 1))) a.full = 1;
@@ -552,20 +564,22 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
 
 bool plan_qsweep_runs(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
                       std::vector<std::pair<std::vector<int>, std::shared_ptr<Args>>>& out, std::string* why,
-                      const std::vector<int>* steps, int step_stride) {
+                      const std::vector<int>* steps, int step_stride, size_t reserve) {
   auto a = std::make_shared<Args>();
-  if (plan_qsweep(f, factors, local_mask, T, B, *a, why, steps, step_stride)) {
+  if (plan_qsweep(f, factors, local_mask, T, B, *a, why, steps, step_stride, reserve)) {
     out.emplace_back(factors, std::move(a));
     return true;
   }
   if (factors.size() < 2) return false;
   const size_t h = factors.size() / 2;
   const std::vector<int> lo(factors.begin(), factors.begin() + h), hi(factors.begin() + h, factors.end());
-  if (!steps) return plan_qsweep_runs(f, lo, local_mask, T, B, out, why) && plan_qsweep_runs(f, hi, local_mask, T, B, out, why);
+  if (!steps)
+    return plan_qsweep_runs(f, lo, local_mask, T, B, out, why, nullptr, 0, reserve) &&
+           plan_qsweep_runs(f, hi, local_mask, T, B, out, why, nullptr, 0, reserve);
   // each piece addresses its records relative to its own first step
   const std::vector<int> slo(steps->begin(), steps->begin() + h), shi(steps->begin() + h, steps->end());
-  return plan_qsweep_runs(f, lo, local_mask, T, B, out, why, &slo, step_stride) &&
-         plan_qsweep_runs(f, hi, local_mask, T, B, out, why, &shi, step_stride);
+  return plan_qsweep_runs(f, lo, local_mask, T, B, out, why, &slo, step_stride, reserve) &&
+         plan_qsweep_runs(f, hi, local_mask, T, B, out, why, &shi, step_stride, reserve);
 }
 
 }  // namespace q

@@ -775,8 +775,16 @@ __device__ __forceinline__ void make_tables(const Args& a, const SmemMap& sm, un
 // starts copying its rows of the CTA's next state or tile, which land while
 // the current one finishes in registers and goes straight back to HBM.
 // ---------------------------------------------------------------------------
+// Slots of one PHASE run whose patterns across the groups take turns: 0, the
+// register bits, the patterns inside the groups, one across.
+template <int B>
+constexpr int kMaxFac = 2 + B + ((1 << lower_bits(B)) - 1 - lower_bits(B)) + ((1 << (B - lower_bits(B))) - 1 - (B - lower_bits(B)));
+
 // D: Args (the tables are made here) or Hdr (they are copied from the image).
-template <typename R, int B, bool FULL, bool EXACT, typename D>
+// LEAN: a thread's phase factors in local memory instead of shared-memory slots,
+// computed on each use, and one copy of the class constants for all warps: the
+// same arithmetic in less shared memory.
+template <typename R, int B, bool FULL, bool EXACT, bool LEAN, typename D>
 __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1, uint32_t stride,
                                             unsigned char* smem_raw) {
   using T2 = typename C2<R>::T;
@@ -805,6 +813,8 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
   OpRec<R>* ops = reinterpret_cast<OpRec<R>*>(at(&SmemMap::ops));
   LayRec* lays = reinterpret_cast<LayRec*>(at(&SmemMap::lays));
   T2* fac = reinterpret_cast<T2*>(at(&SmemMap::fac)) + tid;
+  T2 fac_local[LEAN ? kMaxFac<B> : 1];
+  const int cwarp = LEAN ? 0 : warp;  // whose copy of the class constants
 
   // Per-CTA tables (written by launches that completed before this grid began).
   if constexpr (kImage) {
@@ -866,17 +876,17 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
     // Per-tile phase constants, in this warp's copy: class sums of +-theta_j
     // (units of pi, each term reduced mod 2 in FP64 by the factor build) with
     // the signs of the tile's fixed bits, reduced mod 2 again; a constant class
-    // becomes its phase op's e0.  (The warp barrier keeps a lane from writing
+    // becomes its phase op's e0.  (The first barrier keeps a lane from writing
     // them while another lane still reads the previous tile's.)
     if (new_tile) {
       have = 0;
       const PClass* scls = reinterpret_cast<const PClass*>(at(&SmemMap::cls));
       const PTerm* spt = reinterpret_cast<const PTerm*>(at(&SmemMap::pt));
       const R* thpi = reinterpret_cast<const R*>(at(&SmemMap::thpi));
-      T2* e0s = reinterpret_cast<T2*>(at(&SmemMap::e0s)) + warp * a.n_phase;
-      ClassC<R>* cw = reinterpret_cast<ClassC<R>*>(at(&SmemMap::cw)) + warp * n_cls;
-      __syncwarp();
-      for (int cc = lane; cc < n_cls; cc += 32) {
+      T2* e0s = reinterpret_cast<T2*>(at(&SmemMap::e0s)) + cwarp * a.n_phase;
+      ClassC<R>* cw = reinterpret_cast<ClassC<R>*>(at(&SmemMap::cw)) + cwarp * n_cls;
+      if constexpr (LEAN) __syncthreads(); else __syncwarp();
+      for (int cc = LEAN ? int(tid) : lane; cc < n_cls; cc += LEAN ? NT : 32) {
         const PClass C = scls[cc];
         R acc = R(0);
         for (int t = C.t0; t < C.t0 + C.nt; ++t) acc += flip_sign(thpi[t], uint32_t(__popc(spt[t].rest & base)));
@@ -891,7 +901,7 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
         }
         cw[cc].thr = C.thr;
       }
-      __syncwarp();
+      if constexpr (LEAN) __syncthreads(); else __syncwarp();
     }
 
     const int cur_state = state;
@@ -997,10 +1007,14 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
         if (c.swap) flip_run<R, B, 0>(x, c.swap);
       } else if (op.type == OP_PHASE) {
         const Phase& P = reinterpret_cast<const Phase*>(at(&SmemMap::ph))[op.idx];
-        const ClassC<R>* cw = reinterpret_cast<const ClassC<R>*>(at(&SmemMap::cw)) + warp * n_cls;
-        const T2 e0 = reinterpret_cast<const T2*>(at(&SmemMap::e0s))[warp * a.n_phase + op.idx];
-        phase_op<R, B>(x, P, cw, e0, local_row(), fac + P.fac0 * NT, NT, !((have >> op.idx) & 1u), a.fac_keep != 0);
-        if (a.fac_keep) have |= 1u << op.idx;
+        const ClassC<R>* cw = reinterpret_cast<const ClassC<R>*>(at(&SmemMap::cw)) + cwarp * n_cls;
+        const T2 e0 = reinterpret_cast<const T2*>(at(&SmemMap::e0s))[cwarp * a.n_phase + op.idx];
+        if constexpr (LEAN) {
+          phase_op<R, B>(x, P, cw, e0, local_row(), fac_local, 1, true, false);
+        } else {
+          phase_op<R, B>(x, P, cw, e0, local_row(), fac + P.fac0 * NT, NT, !((have >> op.idx) & 1u), a.fac_keep != 0);
+          if (a.fac_keep) have |= 1u << op.idx;
+        }
       } else if (op.type == OP_BOND) {
         bond_dispatch<R, B>(x, op.ku, T2{ops[oi].c.v[0], ops[oi].c.v[1]});
       } else if (op.type == OP_ROT) {
@@ -1125,14 +1139,15 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
 // register bits, one CTA per SM).  EXACT: a bond sweep applies its scale to more
 // than R's precision.  Rounded, a scale shifts the norm by up to 6e-8 a sweep, all
 // one way: 1.1e-5 over 200 steps of a 20-qubit Heisenberg chain, 1e-8 with it.  (An
-// instantiation of its own: as a branch it cost the MaxCut sweeps 0.5%.)
-template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = false>
+// instantiation of its own: as a branch it cost the MaxCut sweeps 0.5%.)  LEAN:
+// see qsweep_core.
+template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = false, bool LEAN = false>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  qsweep_core<R, B, FULL, EXACT>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
+  qsweep_core<R, B, FULL, EXACT, LEAN>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
 }
 
-template <typename R, int B, bool FULL>
+template <typename R, int B, bool FULL, bool LEAN = false>
 __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_kernel(const __grid_constant__ LevelArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Hdr& a = *reinterpret_cast<Hdr*>(smem_raw + p.prefix_smem);  // the job's header
@@ -1149,7 +1164,7 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
   for (uint32_t w = threadIdx.x; w < sizeof(Hdr) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(&a)[w] = hd[w];
   __syncthreads();
   const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_chunks, BS_BATCH_JOB));
-  qsweep_core<R, B, FULL, false>(a, u, u + 1, 1u, smem_raw);
+  qsweep_core<R, B, FULL, false, LEAN>(a, u, u + 1, 1u, smem_raw);
 }
 
 // One block per image: the template's bytes, then the coefficients of every op
@@ -1210,7 +1225,15 @@ QFn qsweep_fn_t(hs_dtype dt, int B, int tile_bits) {
   if (B == 4 && tb <= 9) return dt == HS_C64 ? qsweep_kernel<float, 4, FULL> : qsweep_kernel<double, 4, FULL>;
   return nullptr;
 }
-QFn qsweep_fn(hs_dtype dt, int B, bool full, int tile_bits, bool exact = false) {
+QFn lean_fn(hs_dtype dt, int B, int tile_bits) {
+  const int tb = tile_bits - B;
+  if (tb < 5 || tb > 9) return nullptr;
+  if (dt == HS_C64 && B == 5) return qsweep_kernel<float, 5, true, 512, false, true>;
+  if (B != 4) return nullptr;
+  return dt == HS_C64 ? qsweep_kernel<float, 4, true, 512, false, true> : qsweep_kernel<double, 4, true, 512, false, true>;
+}
+QFn qsweep_fn(hs_dtype dt, int B, bool full, int tile_bits, bool exact = false, bool lean = false) {
+  if (lean) return lean_fn(dt, B, tile_bits);
   if (exact && !full && dt == HS_C64 && B == 5 && tile_bits >= 10 && tile_bits <= 13)
     return qsweep_kernel<float, 5, false, 256, true>;
   return full ? qsweep_fn_t<true>(dt, B, tile_bits) : qsweep_fn_t<false>(dt, B, tile_bits);
@@ -1222,7 +1245,12 @@ LFn qlevel_fn_t(hs_dtype dt, int B) {
     return B == 5 ? qlevel_kernel<float, 5, FULL> : (B == 4 ? qlevel_kernel<float, 4, FULL> : nullptr);
   return B == 4 ? qlevel_kernel<double, 4, FULL> : nullptr;
 }
-LFn qlevel_fn(hs_dtype dt, int B, bool full) { return full ? qlevel_fn_t<true>(dt, B) : qlevel_fn_t<false>(dt, B); }
+LFn qlevel_fn(hs_dtype dt, int B, bool full, bool lean) {
+  if (!lean) return full ? qlevel_fn_t<true>(dt, B) : qlevel_fn_t<false>(dt, B);
+  if (dt == HS_C64 && B == 5) return qlevel_kernel<float, 5, true, true>;
+  if (B != 4) return nullptr;
+  return dt == HS_C64 ? qlevel_kernel<float, 4, true, true> : qlevel_kernel<double, 4, true, true>;
+}
 
 }  // namespace
 
@@ -1247,7 +1275,13 @@ cudaError_t prepare_qsweep() {
         e = cudaFuncSetAttribute((const void*)qsweep_fn(dts[v], Bs[v], full, 13, true),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute((const void*)qlevel_fn(dts[v], Bs[v], full),
+        e = cudaFuncSetAttribute((const void*)qlevel_fn(dts[v], Bs[v], full, false),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
+      if (e == cudaSuccess && full)
+        e = cudaFuncSetAttribute((const void*)qsweep_fn(dts[v], Bs[v], true, Bs[v] + 8, false, true),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
+      if (e == cudaSuccess && full)
+        e = cudaFuncSetAttribute((const void*)qlevel_fn(dts[v], Bs[v], true, true),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSweepSmemMax));
       if (e != cudaSuccess) return e;
     }
@@ -1307,9 +1341,9 @@ void fill_job(const hs_factors* f, Args& a, void* psi, int n_rhs, int rhs_chunk)
   a.n_chunks = (1 << a.n_tiles_log2) * a.rhs_chunks;
 }
 
-cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
-                          bool pdl, cudaStream_t s) {
-  LFn fn = qlevel_fn(dt, B, full);
+cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, bool lean, int tile_bits, const LevelArgs& L, int64_t ctas,
+                          size_t smem, bool pdl, cudaStream_t s) {
+  LFn fn = qlevel_fn(dt, B, full, lean);
   if (!fn || tile_bits - B < 5 || smem > kSweepSmemMax || ctas <= 0 || ctas >= (int64_t(1) << 31))
     return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
@@ -1330,7 +1364,7 @@ cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const Le
 cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B, bool pdl,
                           cudaStream_t s, const double* rq, const double* cs, int n_terms) {
   const Plan& p = f->plan;
-  QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits, a.exact_scale != 0);
+  QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits, a.exact_scale != 0, a.lean != 0);
   if (!fn || a.tile_bits - B < 5 || a.tile_bits > p.n_qubits) return cudaErrorInvalidValue;
   const size_t smem = qsweep_smem_bytes(a, f->dtype, B);
   if (smem > kSweepSmemMax) return cudaErrorInvalidValue;

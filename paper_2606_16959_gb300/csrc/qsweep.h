@@ -160,6 +160,8 @@ struct Args {
   int n_fac;         // phase factor slots a thread has in shared memory
   int fac_keep;      // 1: every PHASE run has slots of its own (kept for all states of a chunk);
                      // 0: the runs share slots and their factors are computed on each use
+  int lean;          // 1: the instantiation with the factors in local memory (n_fac = 0) and one copy
+                     // of the class constants per CTA
   int last_lay;      // index of the last LAYOUT op
   int free_local;    // 1: the last layout's warp bits are the first one's
   int exact_scale;   // complex64 bonds: 1 takes the instantiation that applies the scale unrounded
@@ -222,8 +224,11 @@ __host__ __device__ __forceinline__ uint32_t across_patterns(uint32_t mu_mask) {
 // spans steps of a time-dependent set whose terms have one record per step:
 // a term record is then addressed (step - steps[0]) * step_stride + kind * m
 // + term, relative to the records of the sweep's first step.
+// reserve: shared memory that a launch needs beside the descriptor's (the header
+// and prefix table of a batch).
 bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
-                 Args& a, std::string* why, const std::vector<int>* steps = nullptr, int step_stride = 0);
+                 Args& a, std::string* why, const std::vector<int>* steps = nullptr, int step_stride = 0,
+                 size_t reserve = 0);
 
 // The tile bits with which HS_METHOD_AUTO takes register sweeps, 0 where it
 // takes the staged ones.
@@ -234,7 +239,7 @@ int auto_tile_bits(const hs_factors* f, int n_rhs, int n_steps);
 // fits.  Returns false if a single factor cannot be expressed.
 bool plan_qsweep_runs(const hs_factors* f, const std::vector<int>& factors, uint32_t local_mask, int T, int B,
                       std::vector<std::pair<std::vector<int>, std::shared_ptr<Args>>>& out, std::string* why,
-                      const std::vector<int>* steps = nullptr, int step_stride = 0);
+                      const std::vector<int>* steps = nullptr, int step_stride = 0, size_t reserve = 0);
 
 // ---------------------------------------------------------------------------
 // Tables in shared memory.  A CTA of a single launch makes them from the
@@ -312,7 +317,7 @@ __host__ __device__ inline SmemMap smem_map(const Args& a, uint32_t e, uint32_t 
     o += (bytes + 15u) & ~15u;
     return at;
   };
-  const uint32_t warps = nt >> 5;
+  const uint32_t copies = a.lean ? 1u : nt >> 5;  // of the class constants
   m.ops = take((e == 8 ? sizeof(OpRec<float>) : sizeof(OpRec<double>)) * a.n_ops);
   m.lays = take(sizeof(LayRec) * a.n_lay);
   m.tabs = take(sizeof(Tab) * a.n_tab);
@@ -324,8 +329,8 @@ __host__ __device__ inline SmemMap smem_map(const Args& a, uint32_t e, uint32_t 
   m.clane = take(48 * 4);
   m.scale = take(16);  // complex64: the scale and what its rounding lost
   m.fac = take(e * nt * a.n_fac);
-  m.e0s = take(e * warps * a.n_phase);
-  m.cw = take(e * warps * a.n_cls);  // a class constant and its mask: the element size
+  m.e0s = take(e * copies * a.n_phase);
+  m.cw = take(e * copies * a.n_cls);  // a class constant and its mask: the element size
   m.total = o;
   return m;
 }
@@ -414,7 +419,7 @@ struct LevelArgs {
 };
 constexpr uint32_t kHdrSmem = 256;
 static_assert(sizeof(Hdr) <= kHdrSmem, "a header and the prefix table do not overlap");
-cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
+cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, bool lean, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
                           bool pdl, cudaStream_t s);
 // rq, cs (optional): term records to use instead of the factor set's own
 // (n_terms of them), for a sweep over steps of a time-dependent set.

@@ -28,7 +28,7 @@ LIB_PATH = os.path.join(_HERE, "_build_debug" if DEBUG_BOUNDS else "_build", "li
 EXPORTS = (
     "hs_build_factors", "hs_build_factors_masks", "hs_evolve", "hs_evolve_ex", "hs_apply_factor",
     "hs_fidelity", "hs_inner_device", "hs_factors_info", "hs_factor_get", "hs_free_factors", "hs_last_error",
-    "hs_plan_factors", "hs_plan_schedule", "hs_evolve_plan", "hs_evolve_td_plan", "hs_inner_batch_noalloc", "hs_autotune",
+    "hs_plan_factors", "hs_plan_schedule", "hs_plan_register", "hs_evolve_plan", "hs_evolve_td_plan", "hs_inner_batch_noalloc", "hs_autotune",
     "hs_batch_create", "hs_batch_launch", "hs_batch_info", "hs_batch_free", "hs_free_factors_async",
     "hs_batch_free_async",
     "hs_dia_from_terms", "hs_dia_from_masks", "hs_dia_create", "hs_spgemm", "hs_spme", "hs_estimate_timesteps",
@@ -92,6 +92,8 @@ def lib() -> ctypes.CDLL:
                                       ip, ip, ip, ip, ip, i64p, i64p, i, i]
         L.hs_plan_schedule.argtypes = [ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64), sz, i, i, i,
                                        i, i, i, i, i, i, ip, ip, ip, ip, ip, i]
+        L.hs_plan_register.argtypes = [ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64),
+                                       ctypes.POINTER(d), sz, i, i, i, i, i, i, i, i, sz, ip, ip, i64p, ip, ip]
         L.hs_evolve_plan.argtypes = [vp, i, i, ctypes.POINTER(EvolveOpts), ip, ip, ip, ip]
         L.hs_evolve_td_plan.argtypes = [vp, i, i, ctypes.POINTER(EvolveOpts), ip, ip, ip, ip]
         L.hs_inner_batch_noalloc.argtypes = [vp, vp, i, i, i, vp, vp]
@@ -485,6 +487,24 @@ def hs_plan_schedule(x, z, n_qubits: int, diag_budget: int, n_steps: int, tile_b
     ip = lambda a: a.ctypes.data_as(ctypes.POINTER(ctypes.c_int))
     _check(lib().hs_plan_schedule(*args, ip(fac), ip(st), ip(sw), na.value))
     return fac, st, sw
+
+
+def hs_plan_register(x, z, coeffs, n_qubits: int, diag_budget: int, n_steps: int, tile_bits: int = 0, reg_bits: int = 0,
+                     order: int = 1, dtype="c64", driven: bool = False, reserve: int = 0) -> dict:
+    """Host-only plan of an evolution by register sweeps (no GPU): launches and shared memory."""
+    xa = np.ascontiguousarray(np.asarray(x, dtype=np.uint64))
+    za = np.ascontiguousarray(np.asarray(z, dtype=np.uint64))
+    ca = np.ascontiguousarray(np.asarray(coeffs, dtype=np.float64))
+    code = HS_C64 if dtype in ("c64", HS_C64) else HS_C128
+    ns, npl, nl, ops, smem = (ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int64())
+    u64 = ctypes.POINTER(ctypes.c_uint64)
+    _check(lib().hs_plan_register(xa.ctypes.data_as(u64), za.ctypes.data_as(u64),
+                                  ca.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), xa.size, int(n_qubits),
+                                  int(diag_budget), int(order), code, int(n_steps), int(tile_bits), int(reg_bits),
+                                  int(bool(driven)), int(reserve), ctypes.byref(ns), ctypes.byref(npl),
+                                  ctypes.byref(smem), ctypes.byref(nl), ctypes.byref(ops)))
+    return {"n_sweeps": ns.value, "n_plain": npl.value, "smem_max": smem.value, "n_lean": nl.value,
+            "ops_max": ops.value}
 
 
 def hs_inner_batch_noalloc(a, b, out, stream=None) -> None:
