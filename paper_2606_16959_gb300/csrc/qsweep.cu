@@ -1173,22 +1173,11 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
 template <typename R>
 __global__ void __launch_bounds__(128) qfill_kernel(const FillRec* recs) {
   using T2 = typename C2<R>::T;
-  __shared__ double sm[4], sp[4];
-  __shared__ int sk[4];
   const FillRec f = recs[blockIdx.x];
   const int tid = threadIdx.x;
   for (uint32_t w = tid; w < f.bytes / 16; w += 128)
     reinterpret_cast<uint4*>(f.img)[w] = reinterpret_cast<const uint4*>(f.tmpl)[w];
   __syncthreads();
-  double m = 1.0, ph = 0.0;
-  int kq = 0;
-  const Records rec{f.rq, f.cs, f.n_terms_g};
-  const OpRec<R>* src = reinterpret_cast<const OpRec<R>*>(f.tmpl + f.ops);
-  OpRec<R>* dst = reinterpret_cast<OpRec<R>*>(f.img + f.ops);
-  for (int oi = tid; oi < f.n_ops; oi += 128) {
-    const Op op = src[oi].op;
-    dst[oi].c = coef_of<R>(op, reinterpret_cast<const int32_t*>(src[oi].c.v), rec, m, ph, kq);
-  }
   const PTerm* pt = reinterpret_cast<const PTerm*>(f.tmpl + f.pt);
   R* thpi = reinterpret_cast<R*>(f.img + f.thpi);
   for (int t = tid; t < f.n_pterm; t += 128) thpi[t] = R(f.rq[4 * HS_BCHK(pt[t].th, f.n_terms_g, BS_REG_TERM) + 3]);
@@ -1197,16 +1186,20 @@ __global__ void __launch_bounds__(128) qfill_kernel(const FillRec* recs) {
   for (int t = 0; t < f.n_tab; ++t)
     for (int e = tid; e < tabs[t].n; e += 128)
       vts[tabs[t].s0 + e] = reinterpret_cast<const T2*>(f.vt)[HS_BCHK(tabs[t].vt0 + e, f.n_vt_g, BS_REG_VT)];
-  sum_scale(m, ph, kq);
-  if ((tid & 31) == 0) {
-    sm[tid >> 5] = m;
-    sp[tid >> 5] = ph;
-    sk[tid >> 5] = kq;
+  // One warp, as in make_tables: the scale's factors then meet in the same order,
+  // and a batch gives the bits of its jobs alone.
+  if (tid >= 32) return;
+  double m = 1.0, ph = 0.0;
+  int kq = 0;
+  const Records rec{f.rq, f.cs, f.n_terms_g};
+  const OpRec<R>* src = reinterpret_cast<const OpRec<R>*>(f.tmpl + f.ops);
+  OpRec<R>* dst = reinterpret_cast<OpRec<R>*>(f.img + f.ops);
+  for (int oi = tid; oi < f.n_ops; oi += 32) {
+    const Op op = src[oi].op;
+    dst[oi].c = coef_of<R>(op, reinterpret_cast<const int32_t*>(src[oi].c.v), rec, m, ph, kq);
   }
-  __syncthreads();
-  if (tid == 0)
-    *reinterpret_cast<T2*>(f.img + f.scale) = scale_of<R>(sm[0] * sm[1] * sm[2] * sm[3], sp[0] + sp[1] + sp[2] + sp[3],
-                                                          sk[0] + sk[1] + sk[2] + sk[3]);
+  sum_scale(m, ph, kq);
+  if (tid == 0) *reinterpret_cast<T2*>(f.img + f.scale) = scale_of<R>(m, ph, kq);
 }
 
 using LFn = void (*)(LevelArgs);
