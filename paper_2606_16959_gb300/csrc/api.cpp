@@ -858,7 +858,7 @@ static int plan_static(const hs_factors* f, int n_rhs, int n_steps, const hs_evo
     return HS_OK;
   }
   for (auto& a : qp)
-    if (a) a->for_staged = 1;
+    if (a) a->exact_scale = f->dtype == HS_C64;
   return HS_OK;
 }
 

@@ -62,7 +62,6 @@ int Images::add(const Args& a) {
   f.n_ops = a.n_ops;
   f.n_tab = a.n_tab;
   f.n_pterm = a.n_pterm;
-  f.exact_scale = a.exact_scale;
   f.ops = 0;
   f.tabs = m.tabs - m.ops;
   f.vts = m.vts - m.ops;

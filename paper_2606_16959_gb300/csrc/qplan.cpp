@@ -556,7 +556,6 @@ bool plan_qsweep(const hs_factors* f, const std::vector<int>& factors, uint32_t 
   for (int form = 0; !ok && form < 3; ++form) ok = fits(form, small ? kSweepSmemDefault : kSweepSmemMax);
   for (int form = 1; !ok && form < 3; ++form) ok = fits(form, kSweepSmemMax);
   if (!ok) return fail("the sweep's tables exceed the shared memory of a CTA");
-  a.exact_scale = c64 && a.n_bond > 0;
   a.full = 0;
   for (int i = 0; i < a.n_ops; ++i)
     if (a.ops[i].type == OP_TAB || (a.ops[i].type == OP_ROT && !(a.ops[i].flags & 1))) a.full = 1;

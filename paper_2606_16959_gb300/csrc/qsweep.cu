@@ -624,7 +624,7 @@ struct Records {
 
 template <typename R>
 __device__ __forceinline__ Coef<R> coef_of(const Op& op, const int32_t* rec, const Records& t, double& m, double& ph,
-                                           int& kq, bool for_staged = false) {
+                                           int& kq, bool exact = false) {
   Coef<R> c{};
   // A fast rotation (y = 0, z = 0): tan(theta') of the factor build's record.
   auto take = [&](int e, R& v) {
@@ -665,7 +665,7 @@ __device__ __forceinline__ Coef<R> coef_of(const Op& op, const int32_t* rec, con
       if (op.flags & 1) {
         const double s2r = sq(cs * c2) + sq(sn * c2) + sq(sn * s2) + sq(cs * s2);
         m *= 1.0 + 0.5 * (0.5 * (r2 + s2r) - 1.0);
-      } else if (!for_staged) {
+      } else if (!exact) {
         m *= r2;
       }
     }
@@ -682,18 +682,17 @@ __device__ __forceinline__ void sum_scale(double& m, double& ph, int& kq) {
   }
 }
 
-// The sweep's scale: rounded to R and, for complex64, what the rounding took off
-// (0 unless `exact`).
+// The sweep's scale rounded to R; lost: what the rounding took off.
 template <typename R>
-__device__ __forceinline__ void write_scale(void* out, double m, double ph, int kq, bool exact) {
+__device__ __forceinline__ typename C2<R>::T scale_of(double m, double ph, int kq,
+                                                      typename C2<R>::T* lost = nullptr) {
   using T2 = typename C2<R>::T;
   const double u0 = ph + 0.5 * double(kq & 3), u = u0 - 2.0 * rint(0.5 * u0);
   double sn, cn;
   sincospi(u, &sn, &cn);
   const T2 c{R(m * cn), R(-m * sn)};
-  T2* o = static_cast<T2*>(out);
-  o[0] = c;
-  if constexpr (sizeof(R) == 4) o[1] = exact ? T2{R(m * cn - double(c.x)), R(-m * sn - double(c.y))} : T2{R(0), R(0)};
+  if (lost) *lost = T2{R(m * cn - double(c.x)), R(-m * sn - double(c.y))};
+  return c;
 }
 
 // The records of op oi of a descriptor.
@@ -754,10 +753,13 @@ __device__ __forceinline__ void make_tables(const Args& a, const SmemMap& sm, un
       int32_t rec[5];
       records_of(a, op, rec);
       ops[oi].op = op;
-      ops[oi].c = coef_of<R>(op, rec, t, m, ph, kq, a.for_staged != 0);
+      ops[oi].c = coef_of<R>(op, rec, t, m, ph, kq, a.exact_scale != 0);
     }
     sum_scale(m, ph, kq);
-    if (tid == 0) write_scale<R>(smem_raw + sm.scale, m, ph, kq, a.exact_scale != 0);
+    if (tid == 0) {
+      T2* out = reinterpret_cast<T2*>(smem_raw + sm.scale);
+      out[0] = scale_of<R>(m, ph, kq, sizeof(T2) == 8 && a.exact_scale ? out + 1 : nullptr);
+    }
   }
 }
 
@@ -1134,14 +1136,12 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
 // FULL: the kernel with the TAB and general-rotation paths; sweeps without
 // them run the lighter instantiation.  NT: threads per CTA the instantiation
 // is built for (2^(tile_bits - B); 512 for 2^14-row complex64 tiles with five
-// register bits, one CTA per SM).  EXACT: a complex scale is applied to more than
-// R's precision.  Rounded, the scale of a bond sweep shifts the norm by up to 6e-8
-// a sweep, all one way: 1.1e-5 over 200 steps of a 20-qubit Heisenberg chain,
-// 1e-8 with it, at the same time.  (The MaxCut sweeps' instantiation is without it:
-// as a branch it cost them 0.5%.  Sweeps without bonds lose nothing there.)  LEAN:
+// register bits, one CTA per SM).  EXACT: a bond sweep applies its scale to more
+// than R's precision.  Rounded, a scale shifts the norm by up to 6e-8 a sweep, all
+// one way: 1.1e-5 over 200 steps of a 20-qubit Heisenberg chain, 1e-8 with it.  (An
+// instantiation of its own: as a branch it cost the MaxCut sweeps 0.5%.)  LEAN:
 // see qsweep_core.
-template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = (FULL || B != 5 || NT != 256),
-          bool LEAN = false>
+template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = false, bool LEAN = false>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   qsweep_core<R, B, FULL, EXACT, LEAN>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
@@ -1164,7 +1164,7 @@ __global__ void __launch_bounds__(B == 5 ? 256 : 512, B == 5 ? 2 : 1) qlevel_ker
   for (uint32_t w = threadIdx.x; w < sizeof(Hdr) / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(&a)[w] = hd[w];
   __syncthreads();
   const uint32_t u = uint32_t(HS_BCHK(blockIdx.x - uint32_t(pref[lo]), a.n_chunks, BS_BATCH_JOB));
-  qsweep_core<R, B, FULL, true, LEAN>(a, u, u + 1, 1u, smem_raw);
+  qsweep_core<R, B, FULL, false, LEAN>(a, u, u + 1, 1u, smem_raw);
 }
 
 // One block per image: the template's bytes, then the coefficients of every op
@@ -1199,7 +1199,7 @@ __global__ void __launch_bounds__(128) qfill_kernel(const FillRec* recs) {
     dst[oi].c = coef_of<R>(op, reinterpret_cast<const int32_t*>(src[oi].c.v), rec, m, ph, kq);
   }
   sum_scale(m, ph, kq);
-  if (tid == 0) write_scale<R>(f.img + f.scale, m, ph, kq, f.exact_scale != 0);
+  if (tid == 0) *reinterpret_cast<T2*>(f.img + f.scale) = scale_of<R>(m, ph, kq);
 }
 
 using LFn = void (*)(LevelArgs);
@@ -1221,9 +1221,9 @@ QFn qsweep_fn_t(hs_dtype dt, int B, int tile_bits) {
 QFn lean_fn(hs_dtype dt, int B, int tile_bits) {
   const int tb = tile_bits - B;
   if (tb < 5 || tb > 9) return nullptr;
-  if (dt == HS_C64 && B == 5) return qsweep_kernel<float, 5, true, 512, true, true>;
+  if (dt == HS_C64 && B == 5) return qsweep_kernel<float, 5, true, 512, false, true>;
   if (B != 4) return nullptr;
-  return dt == HS_C64 ? qsweep_kernel<float, 4, true, 512, true, true> : qsweep_kernel<double, 4, true, 512, true, true>;
+  return dt == HS_C64 ? qsweep_kernel<float, 4, true, 512, false, true> : qsweep_kernel<double, 4, true, 512, false, true>;
 }
 QFn qsweep_fn(hs_dtype dt, int B, bool full, int tile_bits, bool exact = false, bool lean = false) {
   if (lean) return lean_fn(dt, B, tile_bits);

@@ -164,8 +164,7 @@ struct Args {
                      // of the class constants per CTA
   int last_lay;      // index of the last LAYOUT op
   int free_local;    // 1: the last layout's warp bits are the first one's
-  int exact_scale;   // complex64 bonds: the scale is applied unrounded
-  int for_staged;    // the library's choice in place of staged sweeps (see the norm of BOND)
+  int exact_scale;   // complex64 bonds: 1 takes the instantiation that applies the scale unrounded
   int full;          // 1 if a TAB op or a rotation other than tan form occurs (the larger kernel)
   Op ops[kMaxOps];
   Layout lay[kMaxLayouts];
@@ -364,7 +363,7 @@ struct FillRec {
   int64_t n_vt_g;
   int n_terms_g;
   uint32_t bytes;            // of the image
-  int n_ops, n_tab, n_pterm, exact_scale;
+  int n_ops, n_tab, n_pterm;
   uint32_t ops, tabs, vts, pt, thpi, scale;  // byte offsets in the image
 };
 
