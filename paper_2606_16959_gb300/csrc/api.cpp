@@ -87,18 +87,21 @@ int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* 
   const uint64_t all = (1ull << p.n_qubits) - 1;
   for (size_t wi = 0; wi < sw.size(); ++wi) {
     const hs::Sweep& w = sw[wi];
-    // A sweep reads its tables (term records, value tables, factor values) before
-    // it waits for the launch before it.  The first launch waits for all of that
-    // one: it may be the build, or the records or the drive's rebuild, that writes
-    // them.  From the second on every CTA of the launch before has done so.
-    const bool early = wi > 0;
+    // A sweep starts while the launch before it runs, and reads its tables (term
+    // records, value tables, factor values) before it waits for that one.  The
+    // first sweep waits before: the launch before it may be the build, or the
+    // records or the drive's rebuild, that writes them.  (Every CTA of a sweep has
+    // waited when the next one starts, so from the second on they are complete.)
+    // The 10-qubit TFIM quick start: 87.3 us without the wait, 91.0 with an
+    // ordinary launch in place of this one.
+    const bool wait_first = wi == 0;
     cudaError_t e;
     if (qp && (*qp)[wi] && rec) {
       const int st = w.steps.empty() ? 0 : w.steps[0];
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, early, s, rec->rq + size_t(4) * st * rec->stride,
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, wait_first, s, rec->rq + size_t(4) * st * rec->stride,
                                rec->cs + size_t(2) * st * rec->stride, (rec->n_steps - st) * rec->stride);
     } else if (qp && (*qp)[wi]) {
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, early, s);
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, wait_first, s);
     } else if (w.fused) {
       hs::SweepLaunch L;
       L.src = cur;
@@ -111,7 +114,7 @@ int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* 
       L.n_factors = int(w.factors.size());
       for (int i = 0; i < L.n_factors; ++i) L.factors[i] = w.factors[i];
       L.smem_budget = smem_budget;
-      L.pdl = early;
+      L.wait_first = wait_first;
       L.value_tables = value_tables;
       e = hs::launch_sweep(f, L, s);
     } else {

@@ -250,7 +250,7 @@ struct SweepLaunch {
   int n_factors;
   int factors[kMaxSweepFactors];
   size_t smem_budget;  // shared memory the launch may use (sets the number of factor stages)
-  bool pdl;            // launch with programmatic dependent launch
+  bool wait_first;     // the launch before may be what writes the tables
   bool value_tables;   // read factors that have value tables from them instead of staging planes
 };
 cudaError_t launch_sweep(const hs_factors* f, const SweepLaunch& L, cudaStream_t s);
