@@ -1363,6 +1363,15 @@ cudaError_t launch_spmv(const hs_dia* a, const void* x, void* y, int n_rhs, cuda
   return launch_spmv_w<double, 1>(a, x, y, n_rhs, cfg);
 }
 
+// Room for the table, false where there is none: the evolution then takes the
+// diagonals.
+bool alloc_slots(hs_dia* a, size_t ints, cudaStream_t s) {
+  if (pool_malloc(reinterpret_cast<void**>(&a->d_slots), ints * sizeof(int32_t), s) == cudaSuccess) return true;
+  cudaGetLastError();
+  a->d_slots = nullptr;
+  return false;
+}
+
 // The slot table of a matrix whose masks are known, where that at least halves
 // what an evolution reads (made with the matrix: the evolution can be captured).
 int make_slots(hs_dia* a, cudaStream_t s) {
@@ -1389,12 +1398,8 @@ int make_slots(hs_dia* a, cudaStream_t s) {
       t.push_back(has ? int32_t(a->start[size_t(it->second)] + std::min<int64_t>(0, d)) : kNoDiag);
     }
   }
-  cudaError_t e = pool_malloc(reinterpret_cast<void**>(&a->d_slots), t.size() * sizeof(int32_t), s);
-  if (e != cudaSuccess) {
-    a->d_slots = nullptr;
-    return cuda_err(e, "cudaMallocAsync(slot table)");
-  }
-  e = cudaMemcpyAsync(a->d_slots, t.data(), t.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+  if (!alloc_slots(a, t.size(), s)) return HS_OK;
+  cudaError_t e = cudaMemcpyAsync(a->d_slots, t.data(), t.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
   return e == cudaSuccess ? HS_OK : cuda_err(e, "slot table upload");
 }
 
