@@ -75,6 +75,13 @@ bool has_small_table(const Group& G) {
 //     different exponentials to plan: two steps of 17 x 1 Heisenberg 832 / 902.
 //   complex64 bonds, 18 x 4 376 / 258, 20 x 1 792 / 257; 18 x 1 with two bonds
 //     to a factor 163 / 197, hence the line above that size.
+//   Two places above the complex128 line stay staged.  Sets with X at 14 qubits
+//     below 2^17 rows, where the staged sweeps take all tiles at once (ten steps,
+//     staged / register): TFIM 14 x 6 387 / 410, 14 x 7 385 / 411, MaxCut 14 x 6
+//     387 / 396; 14 x 8 426 / 412, and on either side 13 x 12 449 / 385, 15 x 3
+//     674 / 414.  A single Strang step of bonds from 16 qubits to 2^18 rows, three
+//     sweeps either way and five exponentials to plan: 16 x 2 87 / 116, 17 x 1
+//     83 / 121, 18 x 1 161 / 176; 18 x 2 318 / 229, two steps of 16 x 2 168 / 126.
 // A staged sweep re-reads its tile from shared memory for every factor; below
 // these sizes that fits the time the register sweep's tables take to make.
 // Tiles of 2^10 rows (2^11 from 2^20 rows on) give complex128 enough CTAs: 18 x
@@ -120,6 +127,8 @@ int auto_tile_bits(const hs_factors* f, int n_rhs, int n_steps) {
     return rows >= (int64_t(1) << 22) ? 13 : 12;
   }
   if (rows < (p.order > 2 ? int64_t(1) << 18 : int64_t(3) << 15)) return 0;
+  if (flips && n == 14 && rows < (int64_t(1) << 17)) return 0;
+  if (!flips && p.order == 2 && n_steps == 1 && n >= 16 && rows <= (int64_t(1) << 18)) return 0;
   return rows >= (int64_t(1) << 20) ? 11 : 10;
 }
 
