@@ -952,11 +952,13 @@ def time_taylor(job, args, world, rank):
         U, K, ok = hs.hs_spme(H, job.t / r)
         Uc = hs.hs_dia_convert(U, "c64")
         e0, e1 = E(enable_timing=True), E(enable_timing=True)
+        before = hs.hs_kernel_launches()
         e0.record()
         hs.hs_dia_evolve(Uc, work, r)
         e1.record()
+        gathered = hs.hs_kernel_launches() - before == r + 1  # by flip masks: one launch gathers the entries
         hs.hs_inner_device(work, work, out4)
-        info.update(r=r, K=K, converged=ok, D=U.n_diags, H_diags=H.n_diags,
+        info.update(r=r, K=K, converged=ok, D=U.n_diags, H_diags=H.n_diags, by_masks=gathered,
                     S=int(sum(Uc.N - abs(int(d)) for d in Uc.offsets())))
         return (H, U, Uc), e0, e1
 
@@ -1013,6 +1015,26 @@ def oracle_taylor_sample(budget_s=15.0):
                        "single thread; units r x N")
 
 
+def taylor_roofline(n, info, launch_s, hbm, peak_kind, l2_bytes, traffic):
+    """What a step of the propagator reads and writes over its time.  By flip masks it reads the
+    gathered entries, in a plain step the stored diagonals; what fits the L2 stays there from the
+    second step on, and is no share of the HBM rate."""
+    N = 1 << n
+    by_masks = info["by_masks"]
+    # (the terms flip single qubits, so U's masks are those of fewer than K flips)
+    values = 8 * N * sum(math.comb(n, k) for k in range(info["K"])) if by_masks else 8 * info["S"]
+    per_launch = values + 2 * 8 * N
+    achieved = per_launch / launch_s / 1e9
+    out = {"achieved": achieved, "unit": "GB/s", "kernel": "slot_spmv_kernel" if by_masks else "spmv_kernel",
+           "algorithmic_bytes_per_launch": per_launch, "avg_launch_us": launch_s * 1e6}
+    if per_launch <= l2_bytes:
+        return {"bound": "l2", "peak": None, "frac": None, "traffic": None,
+                "hbm_bytes_per_evolution": 8 * info["S"] + 2 * 8 * N, **out}
+    traffic = None if by_masks else traffic
+    return {"bound": "hbm", "peak": hbm, "frac": achieved / hbm, "traffic": traffic, "peak_source": peak_kind, **out,
+            **dram_fields(traffic, launch_s, hbm)}
+
+
 def run_taylor(args, rank, world):
     import torch
     job, desc = taylor_job(args)
@@ -1022,24 +1044,16 @@ def run_taylor(args, rank, world):
     value = res["units"] * K * world / (res["total_ms"] / 1000.0)
     hbm, peak_kind = peaks()
     launch_s = statistics.mean(res["evolve_ms"]) / 1000.0 / max(1, info["r"])
-    # The terms flip single qubits, so U's masks are those of fewer than K flips; where
-    # they are at most half as many as the diagonals a step reads their entries only.
-    masks = sum(math.comb(job.ham.n_qubits, k) for k in range(info["K"]))
-    by_masks = 2 * masks <= info["D"]
-    kernel = "slot_spmv_kernel" if by_masks else "spmv_kernel"
-    per_launch = 8 * (masks * res["N"] if by_masks else info["S"]) + 2 * 8 * res["N"]
-    achieved = per_launch / launch_s / 1e9
-    traffic = profiled_traffic("taylor16", kernel) if not args.qubits and not by_masks else None
+    roofline = taylor_roofline(job.ham.n_qubits, info, launch_s, hbm, peak_kind,
+                               torch.cuda.get_device_properties(0).L2_cache_size,
+                               profiled_traffic("taylor16", "spmv_kernel") if not args.qubits else None)
     cfg = {"workload": "taylor16", "description": desc, "n_qubits": job.ham.n_qubits, "n_terms": len(job.ham.labels),
            "diag_budget": job.budget, "t": job.t, "n_rhs": 1, "H_diags": info["H_diags"], "n_steps": info["r"],
            "U_diags": info["D"], "taylor_terms": info["K"], "l2": "flushed (512 MiB write) before every timed step"}
     line = {"metric": METRIC, "value": value, "unit": METRIC, "n_gpus": world, "steps": K, "warmup": args.warmup,
             "ms_per_step": res["total_ms"] / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "c64", "data": "synthetic", "config": cfg,
-            "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                         "traffic": traffic, "peak_source": peak_kind, "kernel": kernel,
-                         "algorithmic_bytes_per_launch": per_launch, "avg_launch_us": launch_s * 1e6,
-                         **dram_fields(traffic, launch_s, hbm)},
+            "roofline": roofline,
             "e2e": None, "gpu_launches": res["launches"], "clocks": res["clocks"],
             "evolve_ms_per_step": statistics.mean(res["evolve_ms"]), "final_norm2": res["norm2"]}
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
