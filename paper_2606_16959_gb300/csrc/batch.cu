@@ -269,6 +269,7 @@ int upload_tables(hs_batch* b, cudaStream_t s) {
       return hs::report_error(e == cudaErrorMemoryAllocation ? HS_ENOMEM : HS_ECUDA,
                               std::string("batch tables: ") + cudaGetErrorString(e));
     b->uploaded = true;
+    std::vector<hs::q::Args>().swap(b->qdescs);  // (20 KB each)
     return HS_OK;
   }
   if ((e = upload(&b->d_jobs, b->hjobs, s)) != cudaSuccess || (e = upload(&b->d_sweeps, b->hsweeps, s)) != cudaSuccess ||
