@@ -78,30 +78,31 @@ struct StepRecords {
   int n_steps = 0;
 };
 
+// after_writer: the launch before may be what writes the set's tables.  A sweep is
+// launched to start while the launch before it runs, and reads its tables (term
+// records, value tables, factor values) before it waits for that one; the first
+// sweep is then an ordinary launch.  (Every CTA of a sweep has waited when the next
+// one starts, so from the second on they are complete.)  A static set has no need of
+// it: settle_tables stands behind whatever writes its tables.  (Used for every set,
+// the ordinary launch cost the 10-qubit quick start 3.7 of 87.3 us, and a wait at the
+// start of every sweep kernel the 16-qubit chain's 234 launches 9 of 863 us.)
 int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* psi, int n_rhs, int tile_bits,
                    int rhs_block, size_t smem_budget, bool value_tables, void* scratch, cudaStream_t s,
-                   const QPlans* qp = nullptr, int reg_bits = 0, const StepRecords* rec = nullptr) {
+                   bool after_writer, const QPlans* qp = nullptr, int reg_bits = 0, const StepRecords* rec = nullptr) {
   const hs::Plan& p = f->plan;
   void* cur = psi;
   void* other = scratch;
   const uint64_t all = (1ull << p.n_qubits) - 1;
   for (size_t wi = 0; wi < sw.size(); ++wi) {
     const hs::Sweep& w = sw[wi];
-    // A sweep starts while the launch before it runs, and reads its tables (term
-    // records, value tables, factor values) before it waits for that one.  The
-    // first sweep waits before: the launch before it may be the build, or the
-    // records or the drive's rebuild, that writes them.  (Every CTA of a sweep has
-    // waited when the next one starts, so from the second on they are complete.)
-    // The 10-qubit TFIM quick start: 87.3 us without the wait, 91.0 with an
-    // ordinary launch in place of this one.
-    const bool wait_first = wi == 0;
+    const bool pdl = wi > 0 || !after_writer;
     cudaError_t e;
     if (qp && (*qp)[wi] && rec) {
       const int st = w.steps.empty() ? 0 : w.steps[0];
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, wait_first, s, rec->rq + size_t(4) * st * rec->stride,
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, pdl, s, rec->rq + size_t(4) * st * rec->stride,
                                rec->cs + size_t(2) * st * rec->stride, (rec->n_steps - st) * rec->stride);
     } else if (qp && (*qp)[wi]) {
-      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, wait_first, s);
+      e = hs::q::launch_qsweep(f, *(*qp)[wi], cur, cur, n_rhs, reg_bits, pdl, s);
     } else if (w.fused) {
       hs::SweepLaunch L;
       L.src = cur;
@@ -114,7 +115,7 @@ int enqueue_evolve(const hs_factors* f, const std::vector<hs::Sweep>& sw, void* 
       L.n_factors = int(w.factors.size());
       for (int i = 0; i < L.n_factors; ++i) L.factors[i] = w.factors[i];
       L.smem_budget = smem_budget;
-      L.wait_first = wait_first;
+      L.pdl = pdl;
       L.value_tables = value_tables;
       e = hs::launch_sweep(f, L, s);
     } else {
@@ -354,12 +355,20 @@ cudaMemPool_t library_pool() {
   return pools[dev];
 }
 
+// A write to the stream behind the kernels that wrote a static set's tables, so
+// that none of them is the launch a sweep is started early behind (see
+// enqueue_evolve); it begins when they are complete.
+cudaError_t settle_tables(const hs_factors* f, cudaStream_t s) {
+  return f->bin.coeff1 ? cudaSuccess : cudaMemsetAsync(f->bin.fval, 0, sizeof(double), s);
+}
+
 cudaError_t ensure_diagonals(const hs_factors* f, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(f->diag_mu);
   if (!f->diag_pending) return cudaSuccess;
   const hs_build_inputs& b = f->bin;
-  const cudaError_t e = launch_build_split(f, b.tab_groups, b.n_tab_groups, b.row_groups, b.n_row_groups, s);
+  cudaError_t e = launch_build_split(f, b.tab_groups, b.n_tab_groups, b.row_groups, b.n_row_groups, s);
   if (e == cudaSuccess) f->diag_pending = false;
+  if (e == cudaSuccess) e = settle_tables(f, s);
   return e;
 }
 
@@ -574,6 +583,7 @@ int build_impl(const uint64_t* x, const uint64_t* z, const double* coeffs, const
     fp->diag_pending = true;
   else if (e == cudaSuccess)
     e = hs::launch_build_split(fp, bi.tab_groups, bi.n_tab_groups, bi.row_groups, bi.n_row_groups, s);
+  if (e == cudaSuccess) e = hs::settle_tables(fp, s);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(s);
     release(f.release(), s);
@@ -912,6 +922,7 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
   }
   const QPlans* qpp = qp.empty() ? nullptr : &qp;
   const bool scratch_needed = has_plain(sw);
+  const bool driven = f->bin.coeff1 != nullptr;  // (a drive's rebuild may have been the last launch)
   const size_t smem_budget = o.smem_kb > 0 ? size_t(o.smem_kb) * 1024 : hs::kSweepSmemDefault;
   if (o.method != HS_METHOD_REG || scratch_needed) {  // the schedule reads stored diagonals
     cudaError_t e = hs::ensure_diagonals(f, s);
@@ -935,8 +946,8 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
       e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (e != cudaSuccess) { cudaStreamDestroy(cs); return cuda_fail(e, "cudaStreamBeginCapture"); }
       hs::begin_capture_count();
-      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, o.no_tables == 0, nullptr, cs, qpp,
-                              o.reg_bits);
+      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, o.no_tables == 0, nullptr, cs, driven,
+                              qpp, o.reg_bits);
       const uint64_t n_kernels = hs::end_capture_count();
       cudaGraph_t graph = nullptr;
       e = cudaStreamEndCapture(cs, &graph);
@@ -965,7 +976,8 @@ int hs_evolve_ex(const hs_factors* f, void* psi, int n_rhs, int n_steps, const h
     cudaError_t e = hs::pool_malloc(&scratch, state_bytes, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(scratch state)");
   }
-  int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, o.no_tables == 0, scratch, s, qpp, o.reg_bits);
+  int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, o.no_tables == 0, scratch, s, driven, qpp,
+                          o.reg_bits);
   if (scratch) cudaFreeAsync(scratch, s);
   return rc;
 }
@@ -1142,7 +1154,7 @@ int hs_evolve_td(hs_factors* f, void* psi, int n_rhs, const double* drive, int n
       cudaError_t e = hs::launch_sincos_steps(f, f->d_drive, n_steps, const_cast<double*>(rec.cs),
                                               const_cast<double*>(rec.rq), cs);
       if (e != cudaSuccess) return cuda_fail(e, "step records launch");
-      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, tables, nullptr, cs, qpp, o.reg_bits, &rec);
+      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, tables, nullptr, cs, true, qpp, o.reg_bits, &rec);
       if (rc != HS_OK) return rc;
       // The angles and value tables at the last step's drive; the stored
       // diagonals follow when something reads them (diag_pending below).
@@ -1152,7 +1164,7 @@ int hs_evolve_td(hs_factors* f, void* psi, int n_rhs, const double* drive, int n
     for (int k = 0; k < n_steps; ++k) {
       cudaError_t e = enqueue_drive_rebuild(f, f->d_drive + k, diag_groups, n_diag, cs);
       if (e != cudaSuccess) return cuda_fail(e, "drive rebuild");
-      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, tables, scratch, cs, qpp, o.reg_bits);
+      int rc = enqueue_evolve(f, sw, psi, n_rhs, tb, rb, smem_budget, tables, scratch, cs, true, qpp, o.reg_bits);
       if (rc != HS_OK) return rc;
     }
     // Leave every stored value at the last step's drive (register sweeps

@@ -78,7 +78,6 @@ __global__ void __launch_bounds__(256) apply_plain_kernel(const typename C2<R>::
 template <typename R, int ROWS, int RB>
 __global__ void __launch_bounds__(512) sweep_kernel(const __grid_constant__ sweep::SweepArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (a.wait_first) sweep::grid_dependency_wait();
   const uint32_t u0 = blockIdx.x * uint32_t(a.tiles_per_cta);
   const uint32_t u1 = min(uint32_t(a.n_units), u0 + uint32_t(a.tiles_per_cta));
   sweep::sweep_tiles<R, ROWS, RB, RB == 1>(a, u0, u1, smem_raw);
@@ -196,7 +195,6 @@ cudaError_t launch_apply_plain(const hs_factors* f, int g, const void* x, void* 
 cudaError_t launch_sweep(const hs_factors* f, const SweepLaunch& L, cudaStream_t s) {
   const Plan& p = f->plan;
   SweepArgs a;
-  a.wait_first = L.wait_first;
   a.src = L.src;
   a.dst = L.dst;
   a.vals = f->d_vals;
@@ -307,7 +305,7 @@ cudaError_t launch_sweep(const hs_factors* f, const SweepLaunch& L, cudaStream_t
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = L.pdl ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
   if (e == cudaSuccess) note_launches();
   return e;

@@ -189,6 +189,7 @@ struct hs_batch {
   };
   std::vector<Level> levels;
   int max_count = 0;
+  bool driven = false;  // some job's set is time-dependent
   BJob* d_jobs = nullptr;
   BSweep* d_sweeps = nullptr;
   BFac* d_facs = nullptr;
@@ -304,7 +305,7 @@ int enqueue_batch(hs_batch* b, cudaStream_t s) {
   }
   LevelFn fn = b->dtype == HS_C64 ? level_fn<float>(b->rows) : level_fn<double>(b->rows);
   if (!fn) return hs::report_error(HS_EINVAL, "internal: no batch kernel for this tile size");
-  bool early = false;  // (the factor values are complete before the first level reads them)
+  bool early = !b->driven;  // (as hs::enqueue_evolve's first sweep: a drive's rebuild may be the launch before)
   for (const hs_batch::Level& L : b->levels) {
     LevelArgs a{b->d_jobs, b->d_sweeps, b->d_facs, b->d_lvl_sweep, b->d_lvl_prefix, L.off, L.count, b->tile_bits,
                 b->tiles_per_cta};
@@ -547,6 +548,7 @@ extern "C" int hs_batch_create(const hs_batch_job* jobs, size_t n_jobs, const hs
     }
     const int jid = int(hjobs.size());
     const hs_factors* f = J.factors;
+    b->driven = b->driven || f->bin.coeff1;
     hjobs.push_back(BJob{J.psi, f->d_vals, f->d_vt, f->d_slot_u, f->d_slot_tab, f->d_tab_rb, p.N, p.total_elems,
                          p.total_vt, int(p.slot_u.size()), int(p.tab_rb.size()), p.n_qubits, J.n_rhs});
     const int64_t units = (int64_t(1) << (p.n_qubits - T)) * J.n_rhs;

@@ -250,7 +250,7 @@ struct SweepLaunch {
   int n_factors;
   int factors[kMaxSweepFactors];
   size_t smem_budget;  // shared memory the launch may use (sets the number of factor stages)
-  bool wait_first;     // the launch before may be what writes the tables
+  bool pdl;            // launch with programmatic dependent launch
   bool value_tables;   // read factors that have value tables from them instead of staging planes
 };
 cudaError_t launch_sweep(const hs_factors* f, const SweepLaunch& L, cudaStream_t s);
@@ -263,6 +263,9 @@ cudaError_t launch_inner(const void* a, const void* b, int64_t N, hs_dtype dt, d
 
 // Stream-ordered allocation from the library's memory pool (api.cpp).
 cudaError_t pool_malloc(void** ptr, size_t bytes, cudaStream_t s);
+
+// Enqueued behind the kernels that write a static set's tables (api.cpp).
+cudaError_t settle_tables(const hs_factors* f, cudaStream_t s);
 
 // Build the stored diagonals of a set built with HS_BUILD_DEFER_DIAGONALS, on
 // stream s, if they are not built yet (api.cpp).

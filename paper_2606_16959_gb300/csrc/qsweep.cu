@@ -1144,7 +1144,6 @@ __device__ __forceinline__ void qsweep_core(const D& a, uint32_t q0, uint32_t q1
 template <typename R, int B, bool FULL, int NT = (B == 5 ? 256 : 512), bool EXACT = false, bool LEAN = false>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) qsweep_kernel(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (a.wait_first) grid_dependency_wait();
   qsweep_core<R, B, FULL, EXACT, LEAN>(a, blockIdx.x, uint32_t(a.n_chunks), gridDim.x, smem_raw);
 }
 
@@ -1355,8 +1354,8 @@ cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, bool lean, int tile_bit
   return e;
 }
 
-cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B,
-                          bool wait_first, cudaStream_t s, const double* rq, const double* cs, int n_terms) {
+cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B, bool pdl,
+                          cudaStream_t s, const double* rq, const double* cs, int n_terms) {
   const Plan& p = f->plan;
   QFn fn = qsweep_fn(f->dtype, B, a.full != 0, a.tile_bits, a.exact_scale != 0, a.lean != 0);
   if (!fn || a.tile_bits - B < 5 || a.tile_bits > p.n_qubits) return cudaErrorInvalidValue;
@@ -1369,7 +1368,6 @@ cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* d
   const int slots = kSMs * per_sm;
   fill_job(f, a, const_cast<void*>(src), n_rhs, pick_rhs_chunk(int64_t(1) << (p.n_qubits - a.tile_bits), n_rhs, slots));
   a.dst = dst;
-  a.wait_first = wait_first;
   if (rq) {
     a.rq = rq;
     a.cs = cs;
@@ -1384,7 +1382,7 @@ cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* d
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, a);
   if (e == cudaSuccess) note_launches();
   return e;

@@ -138,7 +138,6 @@ struct PTerm {
 };
 
 struct Args {
-  int wait_first;    // 1: wait for the launch before, which may have written the tables, before reading them
   const void* src;
   void* dst;
   const double* cs;  // (cos, sin) per kind and term (FP64)
@@ -422,11 +421,10 @@ constexpr uint32_t kHdrSmem = 256;
 static_assert(sizeof(Hdr) <= kHdrSmem, "a header and the prefix table do not overlap");
 cudaError_t launch_qlevel(hs_dtype dt, int B, bool full, bool lean, int tile_bits, const LevelArgs& L, int64_t ctas, size_t smem,
                           bool pdl, cudaStream_t s);
-// wait_first: the launch before may be what writes the tables.
 // rq, cs (optional): term records to use instead of the factor set's own
 // (n_terms of them), for a sweep over steps of a time-dependent set.
 cudaError_t launch_qsweep(const hs_factors* f, Args& a, const void* src, void* dst, int n_rhs, int B,
-                          bool wait_first, cudaStream_t s, const double* rq = nullptr, const double* cs = nullptr,
+                          bool pdl, cudaStream_t s, const double* rq = nullptr, const double* cs = nullptr,
                           int n_terms = 0);
 cudaError_t prepare_qsweep();
 

@@ -28,7 +28,6 @@ __device__ __forceinline__ void cfma(T2& acc, const T2 v, const T2 x) {
 // Fused tile sweep.
 // ---------------------------------------------------------------------------
 struct SweepArgs {
-  int wait_first;    // 1: wait for the launch before, which may have written the tables, before reading them
   const void* src;
   void* dst;
   const void* vals;
